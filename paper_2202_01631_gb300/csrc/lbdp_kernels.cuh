@@ -276,6 +276,67 @@ __device__ __forceinline__ R psi_ghost_diff(const DevParams& P, const DevPart& q
     return mul_x(PartR<R>::Hk(q), cn);
 }
 
+// The sums of the differences d that the Laplacian and the gradient need, per
+// weight class: sa, sd = sum d over the axis and the diagonal directions,
+// ga, gd = sum c d over them.
+template <class R>
+struct PsiSums {
+    R sa, sd, ga[3], gd[3];
+};
+
+// Component k (0 x, 1 y, 2 z) of c_i for an i known only at run time: two bits
+// per direction, c + 1, in one constant.
+__host__ __device__ constexpr unsigned long long dir_code(int k)
+{
+    unsigned long long t = 0;
+    for (int i = 0; i < 19; ++i) t |= (unsigned long long)((k == 0 ? cx(i) : k == 1 ? cy(i) : cz(i)) + 1) << (2 * i);
+    return t;
+}
+template <int K>
+__device__ __forceinline__ int dir_comp(int i)
+{
+    constexpr unsigned long long t = dir_code(K);
+    return (int)((t >> (2 * i)) & 3ull) - 1;
+}
+
+// The wetting ghosts of fluid node (x, y, z) on its links into particle q (bit
+// i of bits: direction i), added to the sums of the psi differences.  A loop
+// over the links a node has, not over the 18 directions: the lanes of a warp
+// at a sphere's surface hold different links, and a body per direction, taken
+// by whichever lane needs it, made the blocks of kz_fused next to a sphere
+// run twice as long as the rest of the grid (latency of its square root,
+// division and particle loads, 18 times per slot).  Measured on GB300, FP32:
+// kz_fused 201 -> 131 us with one sphere R = 8 in 128^3, 117 -> 70 us in a
+// 75 x 53 x 101 channel with two, 66 -> 42 us in 24^3.
+template <class R>
+__device__ __forceinline__ void psi_ghosts(const DevParams& P, const DevPart& q, int x, int y, int z, unsigned bits,
+                                           PsiSums<R>& s)
+{
+    const R Hk = PartR<R>::Hk(q);
+    if (Hk == (R)0) return;
+    int D[3];
+    int_offset(P, q.g, x, y, z, D);
+    R r0[3];   // x - X
+    link_offset_r<R>(q.g, D, 0, r0);
+    while (bits) {
+        const int i = __ffs((int)bits) - 1;
+        bits &= bits - 1;
+        const R c0 = (R)dir_comp<0>(i), c1 = (R)dir_comp<1>(i), c2 = (R)dir_comp<2>(i);
+        const R r[3] = {fma_x((R)0.5, c0, r0[0]), fma_x((R)0.5, c1, r0[1]), fma_x((R)0.5, c2, r0[2])};
+        const R rn = sqrt(dot_x(r[0], r[1], r[2], r[0], r[1], r[2]));
+        const R gd = mul_x(Hk, dot_x(c0, c1, c2, r[0], r[1], r[2]) / rn);
+        const R ax = i < 7 ? gd : (R)0, dg = i < 7 ? (R)0 : gd;
+        s.sa += ax;
+        s.sd += dg;
+        s.ga[0] = fma_x(c0, ax, s.ga[0]);
+        s.ga[1] = fma_x(c1, ax, s.ga[1]);
+        s.ga[2] = fma_x(c2, ax, s.ga[2]);
+        s.gd[0] = fma_x(c0, dg, s.gd[0]);
+        s.gd[1] = fma_x(c1, dg, s.gd[1]);
+        s.gd[2] = fma_x(c2, dg, s.gd[2]);
+    }
+}
+
 // Equilibrium population i of (rho, u) as its deviation from the rest
 // equilibrium, f_eq - w_i rho0 =
 // w_i [(rho - rho0) + rho (3 c.u + 4.5 (c.u)^2 - 1.5 u^2)], rounding written out.
@@ -321,28 +382,37 @@ __device__ __forceinline__ R phi0_of(const PrmR<R>& Q, R ps)
 // no force: the link-form divergence sums w_i c_i over all 18 directions of a
 // node, and the particle stress sums w_i c_i and w_i r_b x c_i over the
 // boundary links of a sphere, which vanish for the same reason.
+
 template <class R>
-__device__ __forceinline__ void mu_pressure(const PrmR<R>& Q, R ps, const R d[19], R ph, bool want_p, R& mps,
-                                            R& mph, R pt[kPtFields])
+__device__ __forceinline__ PsiSums<R> psi_sums(const R d[19])
 {
+    PsiSums<R> q;
     // the two weight classes summed in two halves each (shorter chains)
-    const R sa = (d[1] + d[2] + d[3]) + (d[4] + d[5] + d[6]);
-    const R sd = ((d[7] + d[8]) + (d[9] + d[10]) + (d[11] + d[12])) +
-                 ((d[13] + d[14]) + (d[15] + d[16]) + (d[17] + d[18]));
-    const R lap = fma_x(sa, (R)(1.0 / 3.0), sd * (R)(1.0 / 6.0));
+    q.sa = (d[1] + d[2] + d[3]) + (d[4] + d[5] + d[6]);
+    q.sd = ((d[7] + d[8]) + (d[9] + d[10]) + (d[11] + d[12])) +
+           ((d[13] + d[14]) + (d[15] + d[16]) + (d[17] + d[18]));
+#pragma unroll
+    for (int a = 0; a < 3; ++a) q.ga[a] = q.gd[a] = (R)0;
     // opposite pairs (j, j + 1), j odd: c_j = -c_{j+1}
-    R ga[3] = {0, 0, 0}, gd[3] = {0, 0, 0};
 #pragma unroll
     for (int j = 1; j < 19; j += 2) {
         const R df = d[j] - d[j + 1];
-        R* acc = j < 7 ? ga : gd;
+        R* acc = j < 7 ? q.ga : q.gd;
         if (cx(j) != 0) acc[0] += cx(j) > 0 ? df : -df;
         if (cy(j) != 0) acc[1] += cy(j) > 0 ? df : -df;
         if (cz(j) != 0) acc[2] += cz(j) > 0 ? df : -df;
     }
-    const R g0 = fma_x(ga[0], (R)(1.0 / 6.0), gd[0] * (R)(1.0 / 12.0));
-    const R g1 = fma_x(ga[1], (R)(1.0 / 6.0), gd[1] * (R)(1.0 / 12.0));
-    const R g2 = fma_x(ga[2], (R)(1.0 / 6.0), gd[2] * (R)(1.0 / 12.0));
+    return q;
+}
+
+template <class R>
+__device__ __forceinline__ void mu_pressure(const PrmR<R>& Q, R ps, const PsiSums<R>& s, R ph, bool want_p, R& mps,
+                                            R& mph, R pt[kPtFields])
+{
+    const R lap = fma_x(s.sa, (R)(1.0 / 3.0), s.sd * (R)(1.0 / 6.0));
+    const R g0 = fma_x(s.ga[0], (R)(1.0 / 6.0), s.gd[0] * (R)(1.0 / 12.0));
+    const R g1 = fma_x(s.ga[1], (R)(1.0 / 6.0), s.gd[1] * (R)(1.0 / 12.0));
+    const R g2 = fma_x(s.ga[2], (R)(1.0 / 6.0), s.gd[2] * (R)(1.0 / 12.0));
     const R t = fma_x(ps, ps, (R)-1);   // psi^2 - 1
     R dphi;
     if (Q.E != (R)0) {
@@ -546,11 +616,14 @@ __device__ __forceinline__ void mup_values(const DevParams& P, const DevPtrs& D,
 {
     using R = typename C::real;
     const PrmR<R>& Q = prm<R>(P);
-    // differences from psi(x): the uniform correction cancels in them
+    // differences from psi(x): the uniform correction cancels in them; 0
+    // towards a wall (neutral) or, until psi_ghosts adds it, a particle
     R d[19];
     uint8_t mk[19];
     const R p0 = (R)a.template get<0>(0);
     d[0] = (R)0;
+    unsigned ids = 0;   // bit i: neighbour i lies inside a particle
+    int lo = 255, hi = 0;
 #pragma unroll
     for (int i = 1; i < 19; ++i) {
         mk[i] = a.mask(i);
@@ -558,12 +631,24 @@ __device__ __forceinline__ void mup_values(const DevParams& P, const DevPtrs& D,
     }
 #pragma unroll
     for (int i = 1; i < 19; ++i) {
-        if (mk[i] == kWallSlot)
-            d[i] = (R)0;
-        else if (mk[i])
-            d[i] = psi_ghost_diff<R>(P, D.parts[mk[i] - 1], x, y, z, i);
+        if (mk[i]) d[i] = (R)0;
+        if (mk[i] && mk[i] != kWallSlot) {
+            ids |= 1u << i;
+            lo = min(lo, (int)mk[i]);
+            hi = max(hi, (int)mk[i]);
+        }
     }
-    mu_pressure<R>(Q, p0 + dps, d, (R)a.template get<1>(0) + dph, P.thermo != 0, mps, mph, pt);
+    PsiSums<R> s = psi_sums<R>(d);
+    for (int k = lo; k <= hi; ++k) {   // the particles next to this node: one, nearly always
+        unsigned bits = ids;
+        if (lo != hi) {
+            bits = 0;
+#pragma unroll
+            for (int i = 1; i < 19; ++i) bits |= mk[i] == k ? 1u << i : 0u;
+        }
+        if (bits) psi_ghosts<R>(P, D.parts[k - 1], x, y, z, bits, s);
+    }
+    mu_pressure<R>(Q, p0 + dps, s, (R)a.template get<1>(0) + dph, P.thermo != 0, mps, mph, pt);
 }
 
 // ---------------------------------------------------------------------------
@@ -1786,7 +1871,7 @@ __global__ void k_mu_now(DevParams P, DevPtrs D)
             neighbours(P, x, y, z, nb);
             R d[19], pt[kPtFields];
             const R ps = gather_psi<R, F>(P, D, psi, x, y, z, nb, d);
-            mu_pressure<R>(prm<R>(P), ps, d, (R)phi[n] + dph, false, mps, mph, pt);
+            mu_pressure<R>(prm<R>(P), ps, psi_sums<R>(d), (R)phi[n] + dph, false, mps, mph, pt);
         }
         ((F*)D.mupsi)[n] = (F)mps;
         ((F*)D.muphi)[n] = (F)mph;
