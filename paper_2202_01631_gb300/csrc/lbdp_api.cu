@@ -143,11 +143,11 @@ DevPtrs cur_ptrs(const lb_handle* h)
     return d;
 }
 
-// z chunk length the size heuristic picks: enough chunks for about six waves
-// of four blocks per SM on 152 SMs, each chunk at least 6 planes long
+// z chunk length of kz_scalars without lb_tune: enough chunks for about six
+// waves of four blocks per SM on 152 SMs, each chunk at least 6 planes long
 // (measured on GB300: 256^3 is fastest with chunks of 12 to 24 planes, 128^3
 // with 6 to 8; shorter chunks repeat more halo planes, fewer blocks leave SMs
-// idle).  lb_tune replaces it with a measured choice.
+// idle).
 int default_planes(const DevParams& P)
 {
     const long long cols = (long long)((P.nx + 31) / 32) * ((P.ny + 7) / 8);
@@ -157,6 +157,42 @@ int default_planes(const DevParams& P)
     if (chunks > max_chunks) chunks = max_chunks;
     if (chunks < 1) chunks = 1;
     return (int)((P.nz + chunks - 1) / chunks);
+}
+
+// z chunk length of kz_fused without lb_tune: the one of least cost under a
+// model of the march.  FP32 arithmetic (halves = 2): a block walks half its
+// chunk's planes in pairs, after about three planes' time to start; 304 blocks
+// run at a time, one alone on its SM in about 0.7 of the time; and the grid
+// ends with its slowest blocks, those beside a sphere above all.  FP64 (halves
+// = 1): the FP64 pipe of an SM is the limit, so the cost is the planes of the
+// blocks an SM gets, plus 1.3 per block for the recomputed halo planes.
+// Measured on GB300 over 1 to 128 planes (us, choice in brackets): FP32 with a
+// sphere 24^3 2 planes 31, 6 planes 44 [1]; 128^3 4 planes 123, 6 110, 8 115,
+// 12 128 [8]; 256^3 8 planes 668, 24 603, 32 597, 64 623 [32]; without one 64^3
+// 2 planes 26, 4 20, 16 31 [4]; 80 x 76 x 84 4 planes 51, 10 42, 24 57 [10];
+// FP64 32^3 1 plane 115, 6 planes 333 [1]; 96^3 4 planes 1062, 8 986, 24 1071 [8].
+int default_fused_planes(const DevParams& P, int halves)
+{
+    const long long cols = (long long)((P.nx + 31) / 32) * ((P.ny + 7) / 8);
+    double best = 1e300;
+    int planes = 1;
+    for (int p = 1; p <= 64 && p <= P.nz; ++p) {
+        const int chunks = (P.nz + p - 1) / p;
+        if ((P.nz + chunks - 1) / chunks != p) continue;   // not the length of equal chunks
+        const long long blocks = cols * chunks;
+        double cost;
+        if (halves == 2) {
+            const double waves = blocks <= 152 ? 0.7 : blocks <= 304 ? 1.0 : blocks <= 608 ? 2.0 : (double)blocks / 304;
+            cost = (waves + (P.np > 0 ? 1.5 : 0.5)) * ((p + 1) / 2 + 3);
+        } else {
+            cost = ((double)((blocks + 151) / 152) + (P.np > 0 ? 0.5 : 0.25)) * (p + 1.3);
+        }
+        if (cost < best) {
+            best = cost;
+            planes = p;
+        }
+    }
+    return planes;
 }
 
 // Grid of a z-marching kernel with chunks of `planes` planes (no empty chunk).
@@ -172,7 +208,8 @@ RowGrid row_grid(const lb_handle* h)
 {
     RowGrid g;
     const int d = default_planes(h->dp);
-    g.zgrid = zm_grid(h->dp, h->zplanes[0] > 0 ? h->zplanes[0] : d);
+    const int halves = h->prm.precision == LB_FP64 ? 1 : 2;
+    g.zgrid = zm_grid(h->dp, h->zplanes[0] > 0 ? h->zplanes[0] : default_fused_planes(h->dp, halves));
     g.zgrid_s = zm_grid(h->dp, h->zplanes[1] > 0 ? h->zplanes[1] : d);
     return g;
 }

@@ -75,7 +75,7 @@ __device__ __forceinline__ bool zm_decode(const DevParams& P, int zc, int bx, in
 template <class C, int ZC>
 __global__ void __launch_bounds__(kZThreads, fused_blocks_per_sm<C>()) kbz_fused(const __grid_constant__ BoxLaunch L)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];   // sizeof(FusedSmem<F>)
+    extern __shared__ __align__(16) unsigned char smem_raw[];   // fused_smem_bytes<C>()
     const int b = blockIdx.y;
     if (b >= L.nbox || L.left[L.base + b] <= 0) return;
     const DevParams& P = L.box[b].P;

@@ -299,17 +299,27 @@ __device__ __forceinline__ int dir_comp(int i)
     return (int)((t >> (2 * i)) & 3ull) - 1;
 }
 
+// 1 / sqrt(a): the CUDA function in FP64; in FP32 the CUDA function and one
+// Newton-Raphson step y (3 - a y^2) / 2, within an ulp.
+__device__ __forceinline__ double inv_sqrt(double a) { return rsqrt(a); }
+__device__ __forceinline__ float inv_sqrt(float a)
+{
+    const float y = rsqrtf(a);
+    return mul_x(y, fma_x(mul_x(-0.5f * a, y), y, 1.5f));
+}
+
 // The wetting ghosts of fluid node (x, y, z) on its links into particle q (bit
 // i of bits: direction i), added to the sums of the psi differences.  A loop
 // over the links a node has, not over the 18 directions: the lanes of a warp
 // at a sphere's surface hold different links, and a body per direction, taken
 // by whichever lane needs it, made the blocks of kz_fused next to a sphere
 // run twice as long as the rest of the grid (latency of its square root,
-// division and particle loads, 18 times per slot).  Measured on GB300, FP32:
-// kz_fused 201 -> 131 us with one sphere R = 8 in 128^3, 117 -> 70 us in a
-// 75 x 53 x 101 channel with two, 66 -> 42 us in 24^3.
-template <class R>
-__device__ __forceinline__ void psi_ghosts(const DevParams& P, const DevPart& q, int x, int y, int z, unsigned bits,
+// division and particle loads, 18 times per slot).  In FP32 two links go
+// through each iteration, for the latency of the inverse square root.
+// Measured on GB300, FP32, loop against unrolled bodies: kz_fused 201 -> 131
+// us with one sphere R = 8 in 128^3, 66 -> 42 us in 24^3.
+template <class R, class Q>
+__device__ __forceinline__ void psi_ghosts(const DevParams& P, const Q& q, int x, int y, int z, unsigned bits,
                                            PsiSums<R>& s)
 {
     const R Hk = PartR<R>::Hk(q);
@@ -318,22 +328,27 @@ __device__ __forceinline__ void psi_ghosts(const DevParams& P, const DevPart& q,
     int_offset(P, q.g, x, y, z, D);
     R r0[3];   // x - X
     link_offset_r<R>(q.g, D, 0, r0);
+    constexpr int U = sizeof(R) == 4 ? 2 : 1;
     while (bits) {
-        const int i = __ffs((int)bits) - 1;
-        bits &= bits - 1;
-        const R c0 = (R)dir_comp<0>(i), c1 = (R)dir_comp<1>(i), c2 = (R)dir_comp<2>(i);
-        const R r[3] = {fma_x((R)0.5, c0, r0[0]), fma_x((R)0.5, c1, r0[1]), fma_x((R)0.5, c2, r0[2])};
-        const R rn = sqrt(dot_x(r[0], r[1], r[2], r[0], r[1], r[2]));
-        const R gd = mul_x(Hk, dot_x(c0, c1, c2, r[0], r[1], r[2]) / rn);
-        const R ax = i < 7 ? gd : (R)0, dg = i < 7 ? (R)0 : gd;
-        s.sa += ax;
-        s.sd += dg;
-        s.ga[0] = fma_x(c0, ax, s.ga[0]);
-        s.ga[1] = fma_x(c1, ax, s.ga[1]);
-        s.ga[2] = fma_x(c2, ax, s.ga[2]);
-        s.gd[0] = fma_x(c0, dg, s.gd[0]);
-        s.gd[1] = fma_x(c1, dg, s.gd[1]);
-        s.gd[2] = fma_x(c2, dg, s.gd[2]);
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            // no link left: direction 0, whose ghost c . n_hat is 0
+            const int i = bits ? __ffs((int)bits) - 1 : 0;
+            bits &= bits - 1;
+            const R c0 = (R)dir_comp<0>(i), c1 = (R)dir_comp<1>(i), c2 = (R)dir_comp<2>(i);
+            const R r[3] = {fma_x((R)0.5, c0, r0[0]), fma_x((R)0.5, c1, r0[1]), fma_x((R)0.5, c2, r0[2])};
+            const R gd = mul_x(mul_x(Hk, dot_x(c0, c1, c2, r[0], r[1], r[2])),
+                               inv_sqrt(dot_x(r[0], r[1], r[2], r[0], r[1], r[2])));
+            const R ax = i < 7 ? gd : (R)0, dg = i < 7 ? (R)0 : gd;
+            s.sa += ax;
+            s.sd += dg;
+            s.ga[0] = fma_x(c0, ax, s.ga[0]);
+            s.ga[1] = fma_x(c1, ax, s.ga[1]);
+            s.ga[2] = fma_x(c2, ax, s.ga[2]);
+            s.gd[0] = fma_x(c0, dg, s.gd[0]);
+            s.gd[1] = fma_x(c1, dg, s.gd[1]);
+            s.gd[2] = fma_x(c2, dg, s.gd[2]);
+        }
     }
 }
 
@@ -351,8 +366,6 @@ __device__ __forceinline__ Real geq_i(int i, Real rho, Real rho0, Real ux, Real 
 
 __device__ __forceinline__ float tanh_r(float v) { return tanhf(v); }
 __device__ __forceinline__ double tanh_r(double v) { return tanh(v); }
-__device__ __forceinline__ float rcp_rn(float v) { return __frcp_rn(v); }
-__device__ __forceinline__ double rcp_rn(double v) { return __drcp_rn(v); }
 
 // phi0 = phi_b + E tanh psi (Eq. free_energy); with E = 0 it is phi_b and tanh
 // is not evaluated.
@@ -583,6 +596,7 @@ struct GAcc {
     int n;
     const uint8_t* mk;
     const F* f[NF];
+    __device__ __forceinline__ const DevPart& part(const DevPtrs& D, int k) const { return D.parts[k]; }
     __device__ __forceinline__ int at(int i) const { return nb[i] >= 0 ? nb[i] : n; }
     __device__ __forceinline__ uint8_t mask(int i) const { return nb[i] >= 0 ? mk[at(i)] : kWallSlot; }
     template <int K>
@@ -646,7 +660,7 @@ __device__ __forceinline__ void mup_values(const DevParams& P, const DevPtrs& D,
 #pragma unroll
             for (int i = 1; i < 19; ++i) bits |= mk[i] == k ? 1u << i : 0u;
         }
-        if (bits) psi_ghosts<R>(P, D.parts[k - 1], x, y, z, bits, s);
+        if (bits) psi_ghosts<R>(P, a.part(D, k - 1), x, y, z, bits, s);
     }
     mu_pressure<R>(Q, p0 + dps, s, (R)a.template get<1>(0) + dph, P.thermo != 0, mps, mph, pt);
 }

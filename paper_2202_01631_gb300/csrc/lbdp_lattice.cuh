@@ -35,6 +35,8 @@ __device__ __forceinline__ double mul_x(double a, double b) { return __dmul_rn(a
 __device__ __forceinline__ float mul_x(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double add_x(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ float add_x(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double rcp_rn(double v) { return __drcp_rn(v); }
+__device__ __forceinline__ float rcp_rn(float v) { return __frcp_rn(v); }
 // a b - c d
 template <class R>
 __device__ __forceinline__ R cross_x(R a, R b, R c, R d)

@@ -74,7 +74,7 @@ struct Ops {
     using F = typename C::fld_t;
 
     static constexpr size_t kLinkSmem = block_rows_bytes<kLinkK>(kPartThreads);
-    static constexpr size_t kFusedSmem = sizeof(FusedSmem<F>);
+    static constexpr size_t kFusedSmem = fused_smem_bytes<C>();
     static constexpr size_t kZScalSmem = sizeof(ScalSmem<F>);
 
     // Opt the kernels that use more than 48 KiB of shared memory in, once per
@@ -263,7 +263,7 @@ struct BOps {
         }
     }
 
-    static size_t smem(int nc) { return nc == 0 ? sizeof(FusedSmem<F>) : sizeof(ScalSmem<F>); }
+    static size_t smem(int nc) { return nc == 0 ? fused_smem_bytes<C>() : sizeof(ScalSmem<F>); }
 
     static cudaError_t prepare()
     {
