@@ -257,7 +257,6 @@ void free_all(lb_handle* h)
         if (h->side.s2) {
             cudaStreamSynchronize(h->side.s2);
             cudaStreamDestroy(h->side.s2);
-            cudaEventDestroy(h->side.pt_done);
             cudaEventDestroy(h->side.links_done);
             cudaEventDestroy(h->side.mark_done);
             h->side.s2 = nullptr;
@@ -1004,7 +1003,6 @@ int lb_create_in(const lb_params* p, lbb_batch* batch, void* region, lb_handle**
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->side.collide_done, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->side.scal_done, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->side.s2, cudaStreamNonBlocking, hi);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->side.pt_done, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->side.links_done, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->side.mark_done, cudaEventDisableTiming);
     }

@@ -325,7 +325,6 @@ int lbb_create(const lbb_params* p, lbb_batch** out)
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->side.collide_done, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->side.scal_done, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&b->side.s2, cudaStreamNonBlocking, hi);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->side.pt_done, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->side.links_done, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->side.mark_done, cudaEventDisableTiming);
     }
@@ -375,7 +374,6 @@ void lbb_destroy(lbb_batch* b)
         cudaStreamSynchronize(b->side.s2);
         cudaStreamDestroy(b->side.s2);
     }
-    if (b->side.pt_done) cudaEventDestroy(b->side.pt_done);
     if (b->side.links_done) cudaEventDestroy(b->side.links_done);
     if (b->side.mark_done) cudaEventDestroy(b->side.mark_done);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);

@@ -17,6 +17,7 @@
 
 #include "lbdp_internal.h"
 #include "lbdp_kernels.cuh"
+#include "lbdp_particles.cuh"
 #include "lbdp_zmarch.cuh"
 
 namespace lbdp {
@@ -98,17 +99,15 @@ __global__ void __launch_bounds__(kZThreads, kScalBlocksPerSM) kbz_scalars(const
 
 // Particle kernels: blockIdx.x = particle * blocks per particle + block.
 template <class C>
-__global__ void __launch_bounds__(kPartThreads, 1) kb_links(const __grid_constant__ BoxLaunch L)
+__global__ void __launch_bounds__(kPartThreads, part_blocks_per_sm<C>()) kb_links(const __grid_constant__ BoxLaunch L)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];   // block_rows_bytes<kLinkK>(kPartThreads)
-    __shared__ DevPart sp;
-    __shared__ bool last;
+    __shared__ LinkSmem<typename C::real> sm;
     const int b = blockIdx.y;
     if (b >= L.nbox || L.left[L.base + b] <= 0) return;
     const DevParams& P = L.box[b].P;
     const int p = blockIdx.x / P.nb1, bi = blockIdx.x % P.nb1;
     if (p >= P.np) return;
-    links_block<C>(P, L.box[b].D[L.par], p, bi, P.nb1, (double*)smem_raw, sp, last);
+    links_block<C>(P, L.box[b].D[L.par], p, bi, P.nb1, sm);
 }
 
 // Stress and force next to the particles, boundary collide-stream and
@@ -116,46 +115,50 @@ __global__ void __launch_bounds__(kPartThreads, 1) kb_links(const __grid_constan
 template <class C>
 __global__ void __launch_bounds__(kPartThreads) kb_pt_part(const __grid_constant__ BoxLaunch L)
 {
+    __shared__ NodeList list;
     const int b = blockIdx.y;
     if (b >= L.nbox || L.left[L.base + b] <= 0) return;
     const DevParams& P = L.box[b].P;
     const int nb = pt_part_blocks(P);
     const int p = blockIdx.x / nb, bi = blockIdx.x % nb;
     if (p >= P.np) return;
-    pt_part_block<C>(P, L.box[b].D[L.par], p, bi, nb);
+    pt_part_block<C>(P, L.box[b].D[L.par], p, bi, nb, list);
 }
 
 template <class C>
 __global__ void __launch_bounds__(kPartThreads) kb_f_part(const __grid_constant__ BoxLaunch L)
 {
+    __shared__ NodeList list;
     const int b = blockIdx.y;
     if (b >= L.nbox || L.left[L.base + b] <= 0) return;
     const DevParams& P = L.box[b].P;
     const int p = blockIdx.x / P.nb1, bi = blockIdx.x % P.nb1;
     if (p >= P.np) return;
-    f_part_block<C>(P, L.box[b].D[L.par], p, bi, P.nb1);
+    f_part_block<C>(P, L.box[b].D[L.par], p, bi, P.nb1, list);
 }
 
 template <class C>
-__global__ void __launch_bounds__(kPartThreads) kb_collide_particles(const __grid_constant__ BoxLaunch L)
+__global__ void __launch_bounds__(kPartThreads, part_blocks_per_sm<C>()) kb_collide_particles(const __grid_constant__ BoxLaunch L)
 {
+    __shared__ ColSmem<typename C::real> sm;
     const int b = blockIdx.y;
     if (b >= L.nbox || L.left[L.base + b] <= 0) return;
     const DevParams& P = L.box[b].P;
     const int p = blockIdx.x / P.nb1, bi = blockIdx.x % P.nb1;
     if (p >= P.np) return;
-    collide_particles_block<C>(P, L.box[b].D[L.par], p, bi, P.nb1);
+    collide_particles_block<C>(P, L.box[b].D[L.par], p, bi, P.nb1, sm);
 }
 
 template <class C>
-__global__ void __launch_bounds__(kPartThreads) kb_scalars_particles(const __grid_constant__ BoxLaunch L)
+__global__ void __launch_bounds__(kPartThreads, part_blocks_per_sm<C>()) kb_scalars_particles(const __grid_constant__ BoxLaunch L)
 {
+    __shared__ NodeList list;
     const int b = blockIdx.y;
     if (b >= L.nbox || L.left[L.base + b] <= 0) return;
     const DevParams& P = L.box[b].P;
     const int p = blockIdx.x / P.nb1, bi = blockIdx.x % P.nb1;
     if (p >= P.np) return;
-    scalars_particles_block<C>(P, L.box[b].D[L.par], p, bi, P.nb1);
+    scalars_particles_block<C>(P, L.box[b].D[L.par], p, bi, P.nb1, list);
 }
 
 template <class C>

@@ -39,7 +39,7 @@ struct SideStream {
     cudaStream_t s;
     cudaEvent_t fork, bnd_done, collide_done, scal_done;
     cudaStream_t s2;   // the link sums and the new mask
-    cudaEvent_t pt_done, links_done, mark_done;
+    cudaEvent_t links_done, mark_done;
     int prio;   // the stream's priority, also given to each of its launches as an attribute
 };
 

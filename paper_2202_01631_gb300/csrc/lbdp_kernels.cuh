@@ -143,28 +143,6 @@ __device__ __forceinline__ R cdot(int i, R a, R b, R c)
     return ta + tb + tc;
 }
 
-// Isotropic gradient of phi at a fluid node, 3 sum_i w_i c_i phi(x+c_i), with
-// the node's own value standing in for solid and wall neighbours.
-template <class R, class Fld>
-__device__ __forceinline__ void grad_phi_at(const int nb[19], const Fld* phi, const uint8_t* mask, R own, R dphi,
-                                            R g[3])
-{
-    g[0] = g[1] = g[2] = (R)0;
-#pragma unroll
-    for (int i = 1; i < 19; ++i) {
-        int m = nb[i];
-        // differences from the node's own value (sum_i w_i c_i = 0)
-        const R v = (m < 0 || mask[m]) ? (R)0 : add_x((R)phi[m] + dphi, -own);
-        const R w = wgt_r<R>(i);
-        if (cx(i) != 0) g[0] = fma_x(cx(i) > 0 ? w : -w, v, g[0]);
-        if (cy(i) != 0) g[1] = fma_x(cy(i) > 0 ? w : -w, v, g[1]);
-        if (cz(i) != 0) g[2] = fma_x(cz(i) > 0 ? w : -w, v, g[2]);
-    }
-    g[0] = mul_x(g[0], (R)3);
-    g[1] = mul_x(g[1], (R)3);
-    g[2] = mul_x(g[2], (R)3);
-}
-
 // ---------------------------------------------------------------------------
 // geometric decisions.  The oracle takes them in FP64 from exact offsets
 // (|x - X|^2 < R^2 for solid nodes, m . r <= 0 for the cap side).  Here they
@@ -201,23 +179,6 @@ __device__ __forceinline__ bool solid_test(const Geo& g, const int D[3], float R
     return dot3_rn(e, e) < R2;
 }
 
-// m . r <= 0 for r = (x - X) + c_i/2 (i = 0: the node itself), the oracle's
-// decision (Eq. MuJ, Eq. activity: the cap side takes mu_- and produces).
-template <class Q>
-__device__ __forceinline__ bool cap_minus(const Q& q, const Geo& g, const int D[3], int i)
-{
-    const float r0 = ((float)D[0] + 0.5f * (float)cx(i)) - g.fr[0];
-    const float r1 = ((float)D[1] + 0.5f * (float)cy(i)) - g.fr[1];
-    const float r2 = ((float)D[2] + 0.5f * (float)cz(i)) - g.fr[2];
-    const float sd = dot_x(q.mf[0], q.mf[1], q.mf[2], r0, r1, r2);
-    if (sd < -q.smarg) return true;
-    if (sd > q.smarg) return false;
-    const double e[3] = {__dsub_rn(__dadd_rn((double)D[0], 0.5 * cx(i)), g.frd[0]),
-                         __dsub_rn(__dadd_rn((double)D[1], 0.5 * cy(i)), g.frd[1]),
-                         __dsub_rn(__dadd_rn((double)D[2], 0.5 * cz(i)), g.frd[2])};
-    return dot3_rn(q.m, e) <= 0.0;
-}
-
 // Link midpoint offset r_b = (x - X) + c_i/2 in the arithmetic precision:
 // exact in FP64, within 2^-24 (1 + |r|) in FP32.
 template <class R>
@@ -235,29 +196,6 @@ __device__ __forceinline__ void link_offset_r<double>(const Geo& g, const int D[
     r[0] = __dsub_rn(__dadd_rn((double)D[0], 0.5 * cx(i)), g.frd[0]);
     r[1] = __dsub_rn(__dadd_rn((double)D[1], 0.5 * cy(i)), g.frd[1]);
     r[2] = __dsub_rn(__dadd_rn((double)D[2], 0.5 * cz(i)), g.frd[2]);
-}
-
-// Boundary velocity at the midpoint of link x -> x + c_i of particle q:
-// u_b = U + Omega x r + v_s, v_s = mu (1 - n n) . grad phi, mu = mu_- where
-// m.r <= 0 else mu_+ (Eq. MuJ).  Returns r (midpoint offset), u_b and v_s.
-template <class R, class Q>
-__device__ __forceinline__ void link_velocity(const DevParams& P, const Q& q, int x, int y, int z, int i,
-                                              const R gphi[3], R r[3], R ub[3], R vs[3])
-{
-    int D[3];
-    int_offset(P, q.g, x, y, z, D);
-    const R mu = cap_minus(q, q.g, D, i) ? PartR<R>::mu_m(q) : PartR<R>::mu_p(q);
-    link_offset_r<R>(q.g, D, i, r);
-    const R rn = sqrt(dot_x(r[0], r[1], r[2], r[0], r[1], r[2]));
-    const R nh[3] = {r[0] / rn, r[1] / rn, r[2] / rn};
-    const R ng = dot_x(nh[0], nh[1], nh[2], gphi[0], gphi[1], gphi[2]);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) vs[a] = mul_x(mu, fma_x(-nh[a], ng, gphi[a]));
-    const R U0 = PartR<R>::U(q, 0), U1 = PartR<R>::U(q, 1), U2 = PartR<R>::U(q, 2);
-    const R W0 = PartR<R>::W(q, 0), W1 = PartR<R>::W(q, 1), W2 = PartR<R>::W(q, 2);
-    ub[0] = add_x(add_x(U0, cross_x(W1, r[2], W2, r[1])), vs[0]);
-    ub[1] = add_x(add_x(U1, cross_x(W2, r[0], W0, r[2])), vs[1]);
-    ub[2] = add_x(add_x(U2, cross_x(W0, r[1], W1, r[0])), vs[2]);
 }
 
 // Wetting ghost of psi at the solid neighbour x + c_i of fluid node x,
@@ -727,23 +665,6 @@ __device__ __forceinline__ void fdiv_compute(const DevParams& P, const DevPtrs& 
     force[2 * N + n] = (F)Fz;
 }
 
-template <class C>
-__device__ __forceinline__ void fdiv_node(const DevParams& P, const DevPtrs& D, int x, int y, int z)
-{
-    using F = typename C::fld_t;
-    const int n = x + P.nx * (y + P.ny * z);
-    if (D.mask[n]) return;
-    const size_t N = (size_t)P.N;
-    const F* pt = (const F*)D.pt;
-    GAcc<F, kPtFields> a;
-    neighbours(P, x, y, z, a.nb);
-    a.n = n;
-    a.mk = D.mask;
-#pragma unroll
-    for (int k = 0; k < kPtFields; ++k) a.f[k] = pt + k * N;
-    fdiv_compute<C>(P, D, n, a);
-}
-
 // Rotate the unit vector m by the angle |w| about w (Rodrigues):
 //   m' = m cos|w| + (w x m) sin|w|/|w| + w (w . m)(1 - cos|w|)/|w|^2,
 // then renormalise.  For |w| < 0.1 both ratios are their Taylor series in
@@ -899,358 +820,6 @@ static __device__ __noinline__ void particle_update(int3 L3, int3 per3, DevPart*
     }
 }
 
-// ---------------------------------------------------------------------------
-// S5 + S6a: link sums and the implicit velocity update.  Grid (nb1, np): the
-// blocks of a particle split its link box; the last block of the particle (a
-// ticket counter) sums the partials in block order and solves
-//   (Mdiag + zeta) V(t+1) = Mdiag V(t) + [F0; T0]
-// (symmetric positive definite: Cholesky), then stores the new velocity and
-// the position/orientation after the step.
-// ---------------------------------------------------------------------------
-//
-// links_block runs block bi of the nbi blocks of particle p; the block split
-// (and with it the summation order) is the same in the single-box and the
-// batched kernels, so both give identical bits.  smem holds
-// block_rows_bytes<kLinkK>(blockDim.x) bytes; sp and last are block-shared.
-template <class C>
-__device__ __forceinline__ void links_block(const DevParams& P, const DevPtrs& D, int p, int bi, int nbi,
-                                            double* smem, DevPart& sp, bool& last)
-{
-    using R = typename C::real;
-    using F = typename C::fld_t;
-    using S = typename C::pop_t;
-    constexpr int K = kLinkK;
-    if (threadIdx.x == 0) sp = D.parts[p];
-    __syncthreads();
-    const DevPart& q = sp;
-    const PrmR<R>& Q = prm<R>(P);
-    const size_t N = (size_t)P.N;
-    const S* fs = (const S*)D.f_src;
-    const F* psi = (const F*)D.psi_src;
-    const F* phi = (const F*)D.phi_src;
-    const R dps = corr_r<R>(D, 0), dph = corr_r<R>(D, 1);
-    // floor(X) - ceil(R) <= floor(X - R): the box holds every fluid node within
-    // R + 2 of the centre
-    const int o[3] = {q.g.Xi[0] - q.Rc - 2, q.g.Xi[1] - q.Rc - 2, q.g.Xi[2] - q.Rc - 2};
-    const int tot = P.side1[0] * P.side1[1] * P.side1[2];
-    double acc[K];
-#pragma unroll
-    for (int k = 0; k < K; ++k) acc[k] = 0.0;
-    const R zc0 = (R)6 * Q.rho0;
-    for (int t = bi * blockDim.x + threadIdx.x; t < tot; t += nbi * blockDim.x) {
-        int x, y, z;
-        if (!box_node(P, o, P.side1, t, x, y, z)) continue;
-        const int n = x + P.nx * (y + P.ny * z);
-        if (D.mask[n]) continue;
-        int nb[19];
-        neighbours(P, x, y, z, nb);
-        // issue every mask load before deciding anything
-        bool lk[19];
-        bool have = false;
-#pragma unroll
-        for (int i = 1; i < 19; ++i) {
-            lk[i] = nb[i] >= 0 && D.mask[nb[i] >= 0 ? nb[i] : n] == p + 1;
-            have = have || lk[i];
-        }
-        if (!have) continue;
-        // this node has links into particle p: load everything it needs at once
-        // (the populations as deviations g_i = f_i - w_i rho0: their constant
-        // part is added exactly below, so the link terms carry small numbers)
-        R fv[19];
-#pragma unroll
-        for (int i = 1; i < 19; ++i) fv[i] = (R)PopStore<S>::load_dev(fs, (size_t)i * N + n, i, Q.rho0);
-        const R ps = (R)psi[n] + dps, ph = (R)phi[n] + dph;
-        R gphi[3];
-        grad_phi_at<R, F>(nb, phi, D.mask, ph, dph, gphi);
-        R pt[kPtFields] = {0, 0, 0, 0};
-        if (P.thermo) {
-            // the stress the fluid's force used this step
-            const F* ptg = (const F*)D.pt;
-#pragma unroll
-            for (int k = 0; k < kPtFields; ++k) pt[k] = (R)ptg[k * N + n];
-        }
-        R nacc[K];   // this node's links, added to the FP64 sums once
-#pragma unroll
-        for (int k = 0; k < K; ++k) nacc[k] = (R)0;
-        // sum over this node's links of 36 w_i c_i (integers: 2 c_i on an
-        // axis link, c_i on a diagonal one)
-        int wc36[3] = {0, 0, 0};
-#pragma unroll
-        for (int i = 1; i < 19; ++i) {
-            if (!lk[i]) continue;
-            wc36[0] += (i < 7 ? 2 : 1) * cx(i);
-            wc36[1] += (i < 7 ? 2 : 1) * cy(i);
-            wc36[2] += (i < 7 ? 2 : 1) * cz(i);
-            R r[3], ub[3], vs[3];
-            link_velocity<R>(P, q, x, y, z, i, gphi, r, ub, vs);
-            const R fi = fv[i];
-            const R w6 = (R)6 * wgt_r<R>(i);
-            const R c[3] = {(R)cx(i), (R)cy(i), (R)cz(i)};
-            const R cvs = cdot<R>(i, vs[0], vs[1], vs[2]);
-            const R mag = fma_x(-mul_x(w6, Q.rho0), cvs, mul_x((R)2, fi));
-            R dP[3] = {mul_x(c[0], mag), mul_x(c[1], mag), mul_x(c[2], mag)};
-            if (P.thermo) {
-                // chemical stress flux through the link, 6 w_i P(x) . c_i
-                R pc[3];
-                pt_dot_c<R>(i, Q.kappa, pt, pc);
-                dP[0] = fma_x(w6, pc[0], dP[0]);
-                dP[1] = fma_x(w6, pc[1], dP[1]);
-                dP[2] = fma_x(w6, pc[2], dP[2]);
-            }
-            nacc[0] = add_x(nacc[0], dP[0]);
-            nacc[1] = add_x(nacc[1], dP[1]);
-            nacc[2] = add_x(nacc[2], dP[2]);
-            nacc[3] = add_x(nacc[3], cross_x(r[1], dP[2], r[2], dP[1]));
-            nacc[4] = add_x(nacc[4], cross_x(r[2], dP[0], r[0], dP[2]));
-            nacc[5] = add_x(nacc[5], cross_x(r[0], dP[1], r[1], dP[0]));
-            const R g6[6] = {c[0], c[1], c[2], cross_x(r[1], c[2], r[2], c[1]), cross_x(r[2], c[0], r[0], c[2]),
-                             cross_x(r[0], c[1], r[1], c[0])};
-            const R zc = mul_x(zc0, wgt_r<R>(i));
-            int k = 6;
-#pragma unroll
-            for (int a = 0; a < 6; ++a)
-#pragma unroll
-                for (int b = a; b < 6; ++b, ++k) nacc[k] = fma_x(mul_x(zc, g6[a]), g6[b], nacc[k]);
-            // scalar flux into the surface, 6 w g(x) c.u_b (finite
-            // differences) or g(x) c.u_b on the six D3Q7 links (lattice
-            // Boltzmann), with c.u_b = (c, r x c) . V(t+1) + c.v_s
-            const R ws = P.scheme ? (i < 7 ? (R)1 : (R)0) : w6;
-            const R wps = mul_x(ws, ps), wph = mul_x(ws, ph);
-#pragma unroll
-            for (int a = 0; a < 6; ++a) {
-                nacc[kLinkGpsi + a] = fma_x(wps, g6[a], nacc[kLinkGpsi + a]);
-                nacc[kLinkGphi + a] = fma_x(wph, g6[a], nacc[kLinkGphi + a]);
-            }
-            nacc[kLinkGpsi + 6] = fma_x(wps, cvs, nacc[kLinkGpsi + 6]);
-            nacc[kLinkGphi + 6] = fma_x(wph, cvs, nacc[kLinkGphi + 6]);
-        }
-#pragma unroll
-        for (int k = 0; k < K; ++k) acc[k] += (double)nacc[k];
-        // The constant parts of the link momentum -- 2 w_i rho0 c_i of the
-        // bounced populations and 6 w_i (A/4) c_i of the chemical stress, whose
-        // stored isotropic part leaves out the bulk pressure A/4 -- in FP64
-        // from the exact counts: the force (2 rho0 + 1.5 A) sum_i w_i c_i and
-        // its torque about the centre, (x - X) x that force (the c_i / 2 of
-        // each link point is parallel to c_i).  Over the closed surface of a
-        // sphere they cancel; they are kept so that every link counts as in
-        // the definition, next to other spheres too.
-        {
-            const PrmR<double>& Qd = prm<double>(P);
-            const double kc = (2.0 * Qd.rho0 + (P.thermo ? 1.5 * Qd.A : 0.0)) / 36.0;
-            const double fc[3] = {kc * (double)wc36[0], kc * (double)wc36[1], kc * (double)wc36[2]};
-            int Dn[3];
-            int_offset(P, q.g, x, y, z, Dn);
-            const double r0[3] = {__dsub_rn((double)Dn[0], q.g.frd[0]), __dsub_rn((double)Dn[1], q.g.frd[1]),
-                                  __dsub_rn((double)Dn[2], q.g.frd[2])};
-            acc[0] += fc[0];
-            acc[1] += fc[1];
-            acc[2] += fc[2];
-            acc[3] += cross_x(r0[1], fc[2], r0[2], fc[1]);
-            acc[4] += cross_x(r0[2], fc[0], r0[0], fc[2]);
-            acc[5] += cross_x(r0[0], fc[1], r0[1], fc[0]);
-        }
-    }
-    block_sum_rows<K>(acc, smem);
-    double* part = D.link_part + ((size_t)p * kMaxPartBlocks + bi) * K;
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < K; ++k) part[k] = acc[k];
-        __threadfence();
-        last = (atomicAdd(D.link_ticket + p, 1u) == (unsigned)nbi - 1u);
-    }
-    __syncthreads();
-    if (!last) return;
-    // last block of this particle: thread b loads block b's partials; the
-    // row reduction adds them in block order
-    __threadfence();
-    double sum[K];
-#pragma unroll
-    for (int k = 0; k < K; ++k) sum[k] = 0.0;
-    if ((int)threadIdx.x < nbi) {
-        const double* pb = D.link_part + ((size_t)p * kMaxPartBlocks + threadIdx.x) * K;
-#pragma unroll
-        for (int k = 0; k < K; ++k) sum[k] = __ldcg(pb + k);
-    }
-    block_sum_rows<K>(sum, smem);   // the totals stay in smem[0..K-1]
-    if (threadIdx.x >= 32) return;
-    particle_update(make_int3(P.nx, P.ny, P.nz), make_int3(P.per[0], P.per[1], P.per[2]), D.parts, D.link_ticket,
-                    D.err, p, q, smem, smem + 64);   // totals in smem[0..K-1], K <= 64
-}
-
-// ---------------------------------------------------------------------------
-// S3: streaming with bounce-back, BGK collision with Guo forcing
-// ---------------------------------------------------------------------------
-
-// BGK collision with Guo forcing of node n from its streamed populations,
-// given as deviations g_i = f_i - w_i rho0 (FP32 cancellation in the moments
-// would otherwise cost the small velocity its low digits):
-//   rho = rho0 + sum g,  j = sum c g  (sum_i w_i c_i = 0),  u = (j + F/2)/rho,
-//   g_eq = w [(rho - rho0) + rho (3 c.u + 4.5 (c.u)^2 - 1.5 u^2)],
-//   S    = w [3 c.F + 9 (c.u)(c.F) - 3 u.F],
-//   g* = (1 - 1/tau) g + g_eq / tau + (1 - 1/(2 tau)) S.
-// Opposite directions (j, j+1) share c.u and c.F up to sign, so
-//   g_eq/tau + (1 - 1/(2tau)) S = P +- Q  with
-//   P = cu (a cu + b cF) + e,  Q = c cu + d cF,
-// a = 4.5 w rho / tau, b = 9 w (1 - 1/(2 tau)), c = 3 w rho / tau,
-// d = 3 w (1 - 1/(2 tau)), e = w (rho - rho0 - 1.5 rho u^2) / tau
-// - 3 w (1 - 1/(2 tau)) u.F, per weight class.  Writes f_dst (as deviations
-// through the storage) and u.
-template <class C>
-__device__ __forceinline__ void collide_store(const PrmR<typename C::real>& Q, const DevPtrs& D, size_t N, int n,
-                                              const typename C::real (&gl)[19], typename C::real Fx,
-                                              typename C::real Fy, typename C::real Fz)
-{
-    using R = typename C::real;
-    using F = typename C::fld_t;
-    using S = typename C::pop_t;
-    S* fd = (S*)D.f_dst + n;
-    const int NN = (int)N;   // 19 N < 2^31
-    const R rho0 = Q.rho0;
-    R dr = 0, jx = 0, jy = 0, jz = 0;
-#pragma unroll
-    for (int j = 0; j < 19; ++j) {
-        dr += gl[j];
-        if (cx(j) != 0) jx += cx(j) > 0 ? gl[j] : -gl[j];
-        if (cy(j) != 0) jy += cy(j) > 0 ? gl[j] : -gl[j];
-        if (cz(j) != 0) jz += cz(j) > 0 ? gl[j] : -gl[j];
-    }
-    const R rho = rho0 + dr;
-    const R ir = rcp_rn(rho);   // IEEE 1 / rho
-    const R ux = fma_x((R)0.5, Fx, jx) * ir;
-    const R uy = fma_x((R)0.5, Fy, jy) * ir;
-    const R uz = fma_x((R)0.5, Fz, jz) * ir;
-    const R itau = Q.itau, omf = Q.omf, keep = (R)1 - itau;
-    const R uu = ux * ux + uy * uy + uz * uz;
-    const R uF = ux * Fx + uy * Fy + uz * Fz;
-    const R base = (dr - (R)1.5 * rho * uu) * itau;   // (rho - rho0 - 1.5 rho u^2) / tau
-    const R tuF = (R)3 * omf * uF;                    // 3 (1 - 1/(2 tau)) u.F
-    // rest direction: w0 (base - 3 (1 - 1/(2 tau)) u.F)
-    PopStore<S>::store_dev(fd, 0, 0, rho0, fma_x(gl[0], keep, wgt_r<R>(0) * (base - tuF)));
-    const R ri = rho * itau;
-    R ka[2], kc[2], ke[2];
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-        const R w = c == 0 ? wgt_r<R>(1) : wgt_r<R>(7);
-        ka[c] = (R)4.5 * w * ri;
-        kc[c] = (R)3 * w * ri;
-        ke[c] = w * (base - tuF);
-    }
-    const R kb0 = (R)9 * wgt_r<R>(1) * omf, kb1 = (R)9 * wgt_r<R>(7) * omf;
-    const R kd0 = (R)3 * wgt_r<R>(1) * omf, kd1 = (R)3 * wgt_r<R>(7) * omf;
-#pragma unroll
-    for (int j = 1; j < 19; j += 2) {
-        const int c = j < 7 ? 0 : 1;
-        const R cu = cdot<R>(j, ux, uy, uz);
-        const R cF = cdot<R>(j, Fx, Fy, Fz);
-        const R Pp = fma_x(cu, fma_x(ka[c], cu, (c ? kb1 : kb0) * cF), ke[c]);
-        const R Qq = fma_x(kc[c], cu, (c ? kd1 : kd0) * cF);
-        PopStore<S>::store_dev(fd, j * NN, j, rho0, fma_x(gl[j], keep, Pp + Qq));
-        PopStore<S>::store_dev(fd, (j + 1) * NN, j + 1, rho0, fma_x(gl[j + 1], keep, Pp - Qq));
-    }
-    F* u = (F*)D.u + n;
-    u[0] = (F)ux;
-    u[NN] = (F)uy;
-    u[2 * NN] = (F)uz;
-}
-
-// Collide-stream of a fluid node next to a particle (and possibly a wall):
-// halfway bounce-back on wall links, moving bounce-back with
-// u_b = U + Omega x r + v_s on particle links.  Every load of the node is
-// issued before any is used (masks, both candidate sources of each
-// population, phi around the node, the force; then the record of the node's
-// lowest adjacent particle).  nb and q (the masks of the neighbours) come
-// from the caller.
-template <class C>
-__device__ __forceinline__ void collide_boundary_wide(const DevParams& P, const DevPtrs& D, int x, int y, int z,
-                                                      const int (&nb)[19], const uint8_t (&q)[19], int lo)
-{
-    using R = typename C::real;
-    using F = typename C::fld_t;
-    using S = typename C::pop_t;
-    const int n = x + P.nx * (y + P.ny * z);
-    const PrmR<R>& Q = prm<R>(P);
-    const size_t N = (size_t)P.N;
-    const int NN = (int)N;
-    const S* fs = (const S*)D.f_src;
-    const F* force = (const F*)D.force;
-    const F* phi = (const F*)D.phi_src;
-    const R rho0 = Q.rho0;
-    const R dph = corr_r<R>(D, 1);
-    const LinkPart lp = link_part(D.parts[lo - 1]);
-    const R Fx = (R)force[n], Fy = (R)force[NN + n], Fz = (R)force[2 * NN + n];
-    const R phn = (R)phi[n];
-    R fl[19], fo[19], pv[19];
-#pragma unroll
-    for (int j = 0; j < 19; ++j) {
-        const int i = opp(j);
-        const int m = nb[i] >= 0 ? nb[i] : n;
-        fl[j] = (R)PopStore<S>::load_dev(fs, j * NN + (j == 0 ? n : m), j, rho0);
-        fo[j] = j == 0 ? (R)0 : (R)PopStore<S>::load_dev(fs, i * NN + n, i, rho0);
-        pv[j] = j == 0 ? (R)0 : (R)phi[nb[j] >= 0 ? nb[j] : n];
-    }
-    // population j arrives from x - c_j = x + c_i (i = opp(j)); from a wall
-    // or a particle it is the node's own population i, reflected
-#pragma unroll
-    for (int j = 1; j < 19; ++j) {
-        const int i = opp(j);
-        if (nb[i] < 0 || q[i] != 0) fl[j] = fo[j];
-    }
-    // grad phi as grad_phi_at, from the values loaded above
-    R gphi[3] = {0, 0, 0};
-    {
-        const R own = phn + dph;
-#pragma unroll
-        for (int i = 1; i < 19; ++i) {
-            const R v = (nb[i] < 0 || q[i]) ? (R)0 : add_x(pv[i] + dph, -own);
-            const R w = wgt_r<R>(i);
-            if (cx(i) != 0) gphi[0] = fma_x(cx(i) > 0 ? w : -w, v, gphi[0]);
-            if (cy(i) != 0) gphi[1] = fma_x(cy(i) > 0 ? w : -w, v, gphi[1]);
-            if (cz(i) != 0) gphi[2] = fma_x(cz(i) > 0 ? w : -w, v, gphi[2]);
-        }
-        gphi[0] = mul_x(gphi[0], (R)3);
-        gphi[1] = mul_x(gphi[1], (R)3);
-        gphi[2] = mul_x(gphi[2], (R)3);
-    }
-#pragma unroll
-    for (int j = 1; j < 19; ++j) {
-        const int i = opp(j);
-        if (nb[i] < 0 || q[i] == 0) continue;
-        R r[3], ub[3], vs[3];
-        if (q[i] == lo)
-            link_velocity<R>(P, lp, x, y, z, i, gphi, r, ub, vs);
-        else
-            link_velocity<R>(P, D.parts[q[i] - 1], x, y, z, i, gphi, r, ub, vs);
-        const R cub = cdot<R>(i, ub[0], ub[1], ub[2]);
-        fl[j] = fma_x(-((R)6 * wgt_r<R>(i) * rho0), cub, fl[j]);
-    }
-    collide_store<C>(Q, D, N, n, fl, Fx, Fy, Fz);
-}
-
-// Pull sources of every population of node (x, y, z) loaded as deviations
-// into fl (wrapped on periodic axes, clamped to the node itself beyond a wall,
-// where bulk_wall_links replaces them): one memory round trip.
-template <class C>
-__device__ __forceinline__ void pull_loads(const DevParams& P, const DevPtrs& D, int x, int y, int z,
-                                           typename C::real (&fl)[19])
-{
-    using R = typename C::real;
-    using S = typename C::pop_t;
-    const int nx = P.nx, ny = P.ny, sxy = nx * ny;
-    const int NN = (int)P.N;
-    const S* fs = (const S*)D.f_src;
-    const R rho0 = prm<R>(P).rho0;
-    // source x - c_j of population j as xi[1 - c_jx] + yo[1 - c_jy] + zo[1 - c_jz]
-    const int xi[3] = {x > 0 ? x - 1 : (P.per[0] ? nx - 1 : 0), x, x < nx - 1 ? x + 1 : (P.per[0] ? 0 : x)};
-    const int yo[3] = {(y > 0 ? y - 1 : (P.per[1] ? ny - 1 : 0)) * nx, y * nx,
-                       (y < ny - 1 ? y + 1 : (P.per[1] ? 0 : y)) * nx};
-    const int zo[3] = {(z > 0 ? z - 1 : (P.per[2] ? P.nz - 1 : 0)) * sxy, z * sxy,
-                       (z < P.nz - 1 ? z + 1 : (P.per[2] ? 0 : z)) * sxy};
-#pragma unroll
-    for (int j = 0; j < 19; ++j) {
-        const int m = xi[1 - cx(j)] + yo[1 - cy(j)] + zo[1 - cz(j)];
-        fl[j] = (R)PopStore<S>::load_dev(fs, j * NN + m, j, rho0);
-    }
-}
-
 // Halfway bounce-back of a bulk node next to a wall: a link whose source lies
 // beyond a wall brings back the node's own population of the opposite
 // direction.
@@ -1275,58 +844,6 @@ __device__ __forceinline__ void bulk_wall_links(const DevParams& P, const DevPtr
 // ---------------------------------------------------------------------------
 // S4: psi and phi transport, production and sink, one thread per node
 // ---------------------------------------------------------------------------
-// Links of fluid node x into particles (transport): no diffusive flux; the
-// scalars leave with the boundary velocity of the bounce-back rule,
-// c.u_b g(x) -- weighted w_i on the D3Q19 links of the finite-difference
-// scheme, 1 on the six D3Q7 links of the lattice-Boltzmann one; Janus
-// production on the m.(x - X) <= 0 side of each adjacent particle (any of
-// the 18 neighbours).  Out of line (few nodes); adds to the running sums in
-// order.
-template <class R>
-struct LinkSums {
-    R sps, sph, src;
-};
-
-template <class C>
-static __device__ __noinline__ LinkSums<typename C::real> scalars_particle_links(
-    const DevParams& P, const DevPtrs& D, int x, int y, int z, typename C::real ps, typename C::real ph,
-    typename C::real sps, typename C::real sph)
-{
-    using R = typename C::real;
-    using F = typename C::fld_t;
-    const F* phi = (const F*)D.phi_src;
-    const R dph = corr_r<R>(D, 1);
-    int nb[19];
-    neighbours(P, x, y, z, nb);
-    unsigned long long adj = 0ull;
-    R gphi[3];
-    grad_phi_at<R, F>(nb, phi, D.mask, ph, dph, gphi);
-    for (int i = 1; i < 19; ++i) {
-        const int m = nb[i];
-        if (m < 0) continue;
-        const uint8_t mk = D.mask[m];
-        if (!mk) continue;
-        adj |= 1ull << (mk - 1);
-        if (P.scheme && i >= 7) continue;
-        R r[3], ubv[3], vs[3];
-        link_velocity<R>(P, D.parts[mk - 1], x, y, z, i, gphi, r, ubv, vs);
-        const R cub = cdot<R>(i, ubv[0], ubv[1], ubv[2]);
-        const R w = P.scheme ? (R)1 : wgt_r<R>(i);
-        sps = fma_x(w, -mul_x(cub, ps), sps);
-        sph = fma_x(w, -mul_x(cub, ph), sph);
-    }
-    R src = 0;
-    while (adj) {
-        const int k = __ffsll((long long)adj) - 1;
-        adj &= adj - 1;
-        const DevPart& q = D.parts[k];
-        int Di[3];
-        int_offset(P, q.g, x, y, z, Di);
-        if (cap_minus(q, q.g, Di, 0)) src += PartR<R>::alpha(q);
-    }
-    return {sps, sph, src};
-}
-
 // psi and phi side by side: on sm_100-class GPUs two FP32 values go through
 // one packed instruction (each lane rounds as the scalar operation does);
 // FP64 keeps two scalar operations.
@@ -1362,10 +879,11 @@ __device__ __forceinline__ Two<double> add2(Two<double> x, Two<double> y) { retu
 // towards y = x + c_j (j = ibar), after taking M mu(x) from each of the six
 // terms of h_0*:
 //   fluid y: M (mu(y) - mu(x)) - g(y) c_j.u(y) / 2,   otherwise g(x) c_j.u(x) / 2
-// and -g(x) c_j.u_b more on a particle link (scalars_particle_links).
+// and -g(x) c_j.u_b more on a particle link (k_scalars_particles).
 template <class C, bool kBoundary, class A>
 __device__ __forceinline__ void scalars_compute_lb(const DevParams& P, const DevPtrs& D, int x, int y, int z,
-                                                   int n, const A& a, typename C::real dps, typename C::real dph)
+                                                   int n, const A& a, typename C::real dps, typename C::real dph,
+                                                   typename C::real eps, typename C::real eph, typename C::real src)
 {
     using R = typename C::real;
     using F = typename C::fld_t;
@@ -1395,12 +913,12 @@ __device__ __forceinline__ void scalars_compute_lb(const DevParams& P, const Dev
         solid_nb = solid_nb || (mk != 0 && mk != kWallSlot);
     }
     R hn_src = 0;
-    if (solid_nb) {
-        if (!kBoundary) return;   // left to k_scalars_particles
-        const LinkSums<R> l = scalars_particle_links<C>(P, D, x, y, z, ps, ph, sps, sph);
-        sps = l.sps;
-        sph = l.sph;
-        hn_src = l.src;
+    if (kBoundary) {
+        sps = add_x(sps, eps);
+        sph = add_x(sph, eph);
+        hn_src = src;
+    } else if (solid_nb) {
+        return;   // left to k_scalars_particles
     }
     // the stored value plus every increment of the step (correction, fluxes,
     // sink, source) summed first: one rounding of the O(1) field per step
@@ -1412,17 +930,20 @@ __device__ __forceinline__ void scalars_compute_lb(const DevParams& P, const Dev
 }
 
 // Fields of the transport body: 0 psi, 1 phi, 2 mu_psi, 3 mu_phi, 4..6 u.
-// kBoundary: nodes next to a particle are transported here; otherwise they
-// are left to k_scalars_particles.
+// kBoundary: a node next to a particle, whose links there carry eps, eph
+// (before the factor 6 of the finite-difference scheme) and whose production
+// is src; otherwise such nodes are left to k_scalars_particles.
 // dps, dph as for mup_values.
 template <class C, bool kBoundary, class A>
 __device__ __forceinline__ void scalars_compute_c(const DevParams& P, const DevPtrs& D, int x, int y, int z, int n,
-                                                  const A& a, typename C::real dps, typename C::real dph)
+                                                  const A& a, typename C::real dps, typename C::real dph,
+                                                  typename C::real eps = 0, typename C::real eph = 0,
+                                                  typename C::real src = 0)
 {
     using R = typename C::real;
     using F = typename C::fld_t;
     if (P.scheme) {
-        scalars_compute_lb<C, kBoundary>(P, D, x, y, z, n, a, dps, dph);
+        scalars_compute_lb<C, kBoundary>(P, D, x, y, z, n, a, dps, dph, eps, eph, src);
         return;
     }
     const PrmR<R>& Q = prm<R>(P);
@@ -1457,12 +978,12 @@ __device__ __forceinline__ void scalars_compute_c(const DevParams& P, const DevP
     }
     R sps = sg.a, sph = sg.b;
     R hn_src = 0;
-    if (solid_nb) {
-        if (!kBoundary) return;   // left to k_scalars_particles
-        const LinkSums<R> l = scalars_particle_links<C>(P, D, x, y, z, ps, ph, sps, sph);
-        sps = l.sps;
-        sph = l.sph;
-        hn_src = l.src;
+    if (kBoundary) {
+        sps = add_x(sps, eps);
+        sph = add_x(sph, eph);
+        hn_src = src;
+    } else if (solid_nb) {
+        return;   // left to k_scalars_particles
     }
     // the stored value plus every increment of the step (correction, fluxes,
     // sink, source) summed first: one rounding of the O(1) field per step
@@ -1471,35 +992,6 @@ __device__ __forceinline__ void scalars_compute_c(const DevParams& P, const DevP
     const R hn = ph0 + ((fma_x((R)6, sph, dph) - Q.kd * (ph - phi0_of(Q, ps))) + hn_src);
     ((F*)D.psi_dst)[n] = (F)pn;
     ((F*)D.phi_dst)[n] = (F)hn;
-}
-
-template <class C, bool kBoundary = true, class A>
-__device__ __forceinline__ void scalars_compute(const DevParams& P, const DevPtrs& D, int x, int y, int z, int n,
-                                                const A& a)
-{
-    using R = typename C::real;
-    scalars_compute_c<C, kBoundary>(P, D, x, y, z, n, a, corr_r<R>(D, 0), corr_r<R>(D, 1));
-}
-
-template <class C>
-__device__ __forceinline__ void scalars_node(const DevParams& P, const DevPtrs& D, int x, int y, int z)
-{
-    using F = typename C::fld_t;
-    const int n = x + P.nx * (y + P.ny * z);
-    if (D.mask[n]) return;
-    const size_t N = (size_t)P.N;
-    GAcc<F, 7> a;
-    neighbours(P, x, y, z, a.nb);
-    a.n = n;
-    a.mk = D.mask;
-    a.f[0] = (const F*)D.psi_src;
-    a.f[1] = (const F*)D.phi_src;
-    a.f[2] = (const F*)D.mupsi;
-    a.f[3] = (const F*)D.muphi;
-    a.f[4] = (const F*)D.u;
-    a.f[5] = (const F*)D.u + N;
-    a.f[6] = (const F*)D.u + 2 * N;
-    scalars_compute<C>(P, D, x, y, z, n, a);
 }
 
 // ---------------------------------------------------------------------------
@@ -1723,91 +1215,10 @@ __device__ __forceinline__ void cover_apply_block(const DevParams& P, const DevP
 }
 
 // ---------------------------------------------------------------------------
-// particle kernels of the single box: grid (blocks per particle, particles)
-// (the bulk kernels of the single box are in lbdp_zmarch.cuh)
+// covering kernels of the single box: grid (blocks per particle, particles)
+// (the other particle kernels are in lbdp_particles.cuh, the bulk kernels in
+// lbdp_zmarch.cuh)
 // ---------------------------------------------------------------------------
-// Collide-stream of the fluid nodes next to particles, beside the bulk kernel
-// (which leaves them out).  These nodes read the particle records and their
-// neighbours' masks in chains of dependent loads; inside the bulk kernel,
-// under its full memory load and register budget, each such chain would hold
-// its block long after the others finish.  Block (b, p) walks the link box of particle
-// p; a node next to several particles is collided by the lowest of them.
-template <class C>
-__device__ __forceinline__ void collide_particles_block(const DevParams& P, const DevPtrs& D, int p, int bi, int nbi)
-{
-    const DevPart& q = D.parts[p];
-    const int o[3] = {q.g.Xi[0] - q.Rc - 2, q.g.Xi[1] - q.Rc - 2, q.g.Xi[2] - q.Rc - 2};
-    const int tot = P.side1[0] * P.side1[1] * P.side1[2];
-    for (int t = bi * blockDim.x + threadIdx.x; t < tot; t += nbi * blockDim.x) {
-        int x, y, z;
-        if (!box_node(P, o, P.side1, t, x, y, z)) continue;
-        const int n = x + P.nx * (y + P.ny * z);
-        if (D.mask[n] || !D.bflag[n]) continue;
-        int nb[19];
-        neighbours(P, x, y, z, nb);
-        uint8_t qm[19];
-        qm[0] = 0;
-        int lo = 256;
-#pragma unroll
-        for (int i = 1; i < 19; ++i) {
-            qm[i] = nb[i] >= 0 ? D.mask[nb[i]] : (uint8_t)0;
-            if (qm[i] != 0 && qm[i] < lo) lo = qm[i];
-        }
-        if (lo != p + 1) continue;
-        collide_boundary_wide<C>(P, D, x, y, z, nb, qm, lo);
-    }
-}
-
-template <class C>
-__global__ void __launch_bounds__(kPartThreads) k_collide_particles(const __grid_constant__ DevParams P,
-                                                                     const __grid_constant__ DevPtrs D)
-{
-    collide_particles_block<C>(P, D, blockIdx.y, blockIdx.x, gridDim.x);
-}
-
-// Transport of the fluid nodes next to particles, beside kz_scalars (which
-// leaves them out), for the same reason and with the same split as
-// k_collide_particles.
-template <class C>
-__device__ __forceinline__ void scalars_particles_block(const DevParams& P, const DevPtrs& D, int p, int bi, int nbi)
-{
-    const DevPart& q = D.parts[p];
-    const int o[3] = {q.g.Xi[0] - q.Rc - 2, q.g.Xi[1] - q.Rc - 2, q.g.Xi[2] - q.Rc - 2};
-    const int tot = P.side1[0] * P.side1[1] * P.side1[2];
-    for (int t = bi * blockDim.x + threadIdx.x; t < tot; t += nbi * blockDim.x) {
-        int x, y, z;
-        if (!box_node(P, o, P.side1, t, x, y, z)) continue;
-        const int n = x + P.nx * (y + P.ny * z);
-        if (D.mask[n] || !D.bflag[n]) continue;
-        int nb[19];
-        neighbours(P, x, y, z, nb);
-        int lo = 256;
-#pragma unroll
-        for (int i = 1; i < 19; ++i) {
-            const int m = nb[i] >= 0 ? D.mask[nb[i]] : 0;
-            if (m != 0 && m < lo) lo = m;
-        }
-        if (lo != p + 1) continue;
-        scalars_node<C>(P, D, x, y, z);
-    }
-}
-
-template <class C>
-__global__ void __launch_bounds__(kPartThreads) k_scalars_particles(const __grid_constant__ DevParams P,
-                                                                     const __grid_constant__ DevPtrs D)
-{
-    scalars_particles_block<C>(P, D, blockIdx.y, blockIdx.x, gridDim.x);
-}
-
-template <class C>
-__global__ void __launch_bounds__(kPartThreads, 1) k_links(DevParams P, DevPtrs D)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];   // block_rows_bytes<kLinkK>(kPartThreads)
-    __shared__ DevPart sp;
-    __shared__ bool last;
-    links_block<C>(P, D, blockIdx.y, blockIdx.x, gridDim.x, (double*)smem_raw, sp, last);
-}
-
 template <class C>
 __global__ void __launch_bounds__(kPartThreads) k_cover_mark(DevParams P, DevPtrs D)
 {

@@ -63,17 +63,11 @@ inline void side_launch(void (*k)(A...), dim3 grid, size_t smem, const SideStrea
     cudaLaunchKernelEx(&cfg, k, args...);
 }
 
-// Resident blocks per SM the tiled force and transport kernels are given
-// (measured on the 128^3 workload: 5 and 4 beat the 7 and 6 their register
-// counts allow by 5 and 10 us).
-constexpr int kFdivBlocks = 5, kScalBlocks = 4;
-
 template <class C>
 struct Ops {
     using R = typename C::real;
     using F = typename C::fld_t;
 
-    static constexpr size_t kLinkSmem = block_rows_bytes<kLinkK>(kPartThreads);
     static constexpr size_t kFusedSmem = fused_smem_bytes<C>();
     static constexpr size_t kZScalSmem = sizeof(ScalSmem<F>);
 
@@ -86,9 +80,7 @@ struct Ops {
         cudaError_t e = cudaGetDevice(&dev);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
-        e = cudaFuncSetAttribute(k_links<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLinkSmem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(kz_fused<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmem);
+        e = cudaFuncSetAttribute(kz_fused<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFusedSmem);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(kz_scalars<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kZScalSmem);
         if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
@@ -114,14 +106,13 @@ struct Ops {
         const dim3 pg1(P.nb1, P.np), pg2(P.nb2, P.np), pgt = pt_grid(P);
         if (P.np > 0 && side && !ev) {
             cudaEventRecord(side->fork, s);
-            cudaStreamWaitEvent(side->s, side->fork, 0);
-            side_launch(k_pt_part<C>, pgt, 0, side, P, D);
-            cudaEventRecord(side->pt_done, side->s);
-            cudaStreamWaitEvent(side->s2, side->pt_done, 0);
-            side_launch_on(side->s2, k_links<C>, pg1, kLinkSmem, side, P, D);
+            cudaStreamWaitEvent(side->s2, side->fork, 0);
+            side_launch_on(side->s2, k_links<C>, pg1, 0, side, P, D);
             cudaEventRecord(side->links_done, side->s2);
             side_launch_on(side->s2, k_cover_mark<C>, pg2, 0, side, P, D);
             cudaEventRecord(side->mark_done, side->s2);
+            cudaStreamWaitEvent(side->s, side->fork, 0);
+            side_launch(k_pt_part<C>, pgt, 0, side, P, D);
             side_launch(k_f_part<C>, pg1, 0, side, P, D);
             cudaStreamWaitEvent(side->s, side->links_done, 0);
             side_launch(k_collide_particles<C>, pg1, 0, side, P, D);
@@ -145,7 +136,7 @@ struct Ops {
         if (P.np > 0) {
             k_pt_part<C><<<pgt, kPartThreads, 0, s>>>(P, D);
             k_f_part<C><<<pg1, kPartThreads, 0, s>>>(P, D);
-            k_links<C><<<pg1, kPartThreads, kLinkSmem, s>>>(P, D);
+            k_links<C><<<pg1, kPartThreads, 0, s>>>(P, D);
             k_collide_particles<C><<<pg1, kPartThreads, 0, s>>>(P, D);
         }
         if (ev) cudaEventRecord(ev[1], s);
@@ -272,8 +263,6 @@ struct BOps {
         cudaError_t e = cudaGetDevice(&dev);
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
-        e = cudaFuncSetAttribute(kb_links<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)block_rows_bytes<kLinkK>(kPartThreads));
         for (int nc = 0; nc < kNumBatchClasses && e == cudaSuccess; ++nc)
             for (int k = 0; k < kNumBatchCfgs && e == cudaSuccess; ++k)
                 e = cudaFuncSetAttribute((const void*)fn(nc, k), cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -298,7 +287,6 @@ struct BOps {
     {
         cudaError_t e = prepare();
         if (e != cudaSuccess) return e;
-        const size_t lsm = block_rows_bytes<kLinkK>(kPartThreads);
         for (int l = 0; l < nl; ++l) {
             LaunchPlan* L = Ls + l;
             L->L.par = par;   // copied into each launch's parameters at the call
@@ -306,14 +294,13 @@ struct BOps {
                 // the single-box stream order: link sums and the new mask on
                 // s2 beside the force and boundary collide on s
                 cudaEventRecord(side->fork, s);
-                cudaStreamWaitEvent(side->s, side->fork, 0);
-                side_launch(kb_pt_part<C>, L->ptg, 0, side, L->L);
-                cudaEventRecord(side->pt_done, side->s);
-                cudaStreamWaitEvent(side->s2, side->pt_done, 0);
-                side_launch_on(side->s2, kb_links<C>, L->link, lsm, side, L->L);
+                cudaStreamWaitEvent(side->s2, side->fork, 0);
+                side_launch_on(side->s2, kb_links<C>, L->link, 0, side, L->L);
                 cudaEventRecord(side->links_done, side->s2);
                 side_launch_on(side->s2, kb_cover_mark<C>, L->cover, 0, side, L->L);
                 cudaEventRecord(side->mark_done, side->s2);
+                cudaStreamWaitEvent(side->s, side->fork, 0);
+                side_launch(kb_pt_part<C>, L->ptg, 0, side, L->L);
                 side_launch(kb_f_part<C>, L->link, 0, side, L->L);
                 cudaStreamWaitEvent(side->s, side->links_done, 0);
                 side_launch(kb_collide_particles<C>, L->link, 0, side, L->L);
@@ -331,7 +318,7 @@ struct BOps {
             } else {
                 kb_pt_part<C><<<L->ptg, kPartThreads, 0, s>>>(L->L);
                 kb_f_part<C><<<L->link, kPartThreads, 0, s>>>(L->L);
-                kb_links<C><<<L->link, kPartThreads, lsm, s>>>(L->L);
+                kb_links<C><<<L->link, kPartThreads, 0, s>>>(L->L);
                 kb_collide_particles<C><<<L->link, kPartThreads, 0, s>>>(L->L);
                 if ((e = node(0, cfg[0], L, s)) != cudaSuccess) return e;
                 if ((e = node(1, cfg[1], L, s)) != cudaSuccess) return e;

@@ -1112,105 +1112,4 @@ __global__ void __launch_bounds__(kZThreads, kScalBlocksPerSM) kz_scalars(const 
     kz_scalars_run<C>(P, D, blockIdx.x * kZX, blockIdx.y * kZY, z0, nt, smem_raw);
 }
 
-// ---------------------------------------------------------------------------
-// the pressure tensor and force next to particles, for the side stream
-// ---------------------------------------------------------------------------
-// P at every fluid node of the link box of particle p grown by one node (the
-// boundary nodes and all their neighbours), into the pressure-tensor array.
-// Nodes in two such boxes are written twice with the same values.
-__device__ __forceinline__ void pt_box(const DevParams& P, const DevPart& q, int o[3], int s[3])
-{
-    const int L[3] = {P.nx, P.ny, P.nz};
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        o[a] = q.g.Xi[a] - q.Rc - 3;
-        s[a] = P.side1[a] + 2;
-        if (P.per[a] && s[a] > L[a]) s[a] = L[a];
-    }
-}
-
-// Blocks per particle of k_pt_part (about one node of the box per thread).
-__host__ __device__ inline int pt_part_blocks(const DevParams& P)
-{
-    long long t = 1;
-    const int L[3] = {P.nx, P.ny, P.nz};
-    for (int a = 0; a < 3; ++a) {
-        int s = P.side1[a] + 2;
-        if (P.per[a] && s > L[a]) s = L[a];
-        t *= s;
-    }
-    const long long b = (t + kPartThreads - 1) / kPartThreads;
-    return (int)(b < 1 ? 1 : (b > kMaxPartBlocks ? kMaxPartBlocks : b));
-}
-
-// Block bi of the nbi blocks of particle p.
-template <class C>
-__device__ __forceinline__ void pt_part_block(const DevParams& P, const DevPtrs& D, int p, int bi, int nbi)
-{
-    using R = typename C::real;
-    using F = typename C::fld_t;
-    if (!P.thermo) return;
-    int o[3], sd[3];
-    pt_box(P, D.parts[p], o, sd);
-    const int tot = sd[0] * sd[1] * sd[2];
-    const size_t N = (size_t)P.N;
-    for (int t = bi * blockDim.x + threadIdx.x; t < tot; t += nbi * blockDim.x) {
-        int x, y, z;
-        if (!box_node(P, o, sd, t, x, y, z)) continue;
-        const int n = x + P.nx * (y + P.ny * z);
-        if (D.mask[n]) continue;
-        GAcc<F, 2> a;
-        neighbours(P, x, y, z, a.nb);
-        a.n = n;
-        a.mk = D.mask;
-        a.f[0] = (const F*)D.psi_src;
-        a.f[1] = (const F*)D.phi_src;
-        R mps, mph, pt[kPtFields];
-        mup_values<C>(P, D, x, y, z, a, corr_r<R>(D, 0), corr_r<R>(D, 1), mps, mph, pt);
-        F* ptg = (F*)D.pt;
-#pragma unroll
-        for (int k = 0; k < kPtFields; ++k) ptg[k * N + n] = (F)pt[k];
-    }
-}
-
-template <class C>
-__global__ void __launch_bounds__(kPartThreads) k_pt_part(const __grid_constant__ DevParams P,
-                                                           const __grid_constant__ DevPtrs D)
-{
-    pt_part_block<C>(P, D, blockIdx.y, blockIdx.x, gridDim.x);
-}
-
-// F at the fluid nodes next to particle p (those whose lowest adjacent
-// particle is p, as in k_collide_particles), into the force array.
-template <class C>
-__device__ __forceinline__ void f_part_block(const DevParams& P, const DevPtrs& D, int p, int bi, int nbi)
-{
-    const DevPart& q = D.parts[p];
-    const int o[3] = {q.g.Xi[0] - q.Rc - 2, q.g.Xi[1] - q.Rc - 2, q.g.Xi[2] - q.Rc - 2};
-    const int tot = P.side1[0] * P.side1[1] * P.side1[2];
-    for (int t = bi * blockDim.x + threadIdx.x; t < tot; t += nbi * blockDim.x) {
-        int x, y, z;
-        if (!box_node(P, o, P.side1, t, x, y, z)) continue;
-        const int n = x + P.nx * (y + P.ny * z);
-        if (D.mask[n] || !D.bflag[n]) continue;
-        int nb[19];
-        neighbours(P, x, y, z, nb);
-        int lo = 256;
-#pragma unroll
-        for (int i = 1; i < 19; ++i) {
-            const int m = nb[i] >= 0 ? D.mask[nb[i]] : 0;
-            if (m != 0 && m < lo) lo = m;
-        }
-        if (lo != p + 1) continue;
-        fdiv_node<C>(P, D, x, y, z);
-    }
-}
-
-template <class C>
-__global__ void __launch_bounds__(kPartThreads) k_f_part(const __grid_constant__ DevParams P,
-                                                          const __grid_constant__ DevPtrs D)
-{
-    f_part_block<C>(P, D, blockIdx.y, blockIdx.x, gridDim.x);
-}
-
 }  // namespace lbdp
