@@ -111,6 +111,7 @@ DevPtrs ptrs(const lb_handle* h, int src)
     d.phi_dst = h->phi[dst];
     d.mupsi = h->mupsi;
     d.muphi = h->muphi;
+    d.mu = h->mupsi;   // mupsi and muphi follow one another in the region: room for both of every node
     d.u = h->u;
     d.mask = h->mask[src];
     d.mask_next = h->mask[dst];
@@ -141,22 +142,6 @@ DevPtrs cur_ptrs(const lb_handle* h)
     d.phi_dst = h->phi[h->cur];
     d.mask_next = h->mask[h->cur];
     return d;
-}
-
-// z chunk length of kz_scalars without lb_tune: enough chunks for about six
-// waves of four blocks per SM on 152 SMs, each chunk at least 6 planes long
-// (measured on GB300: 256^3 is fastest with chunks of 12 to 24 planes, 128^3
-// with 6 to 8; shorter chunks repeat more halo planes, fewer blocks leave SMs
-// idle).
-int default_planes(const DevParams& P)
-{
-    const long long cols = (long long)((P.nx + 31) / 32) * ((P.ny + 7) / 8);
-    const long long target = 152LL * 4 * 6;
-    long long chunks = (target + cols - 1) / cols;
-    const long long max_chunks = P.nz / 6 > 1 ? P.nz / 6 : 1;
-    if (chunks > max_chunks) chunks = max_chunks;
-    if (chunks < 1) chunks = 1;
-    return (int)((P.nz + chunks - 1) / chunks);
 }
 
 // z chunk length of kz_fused without lb_tune: the one of least cost under a
@@ -195,6 +180,32 @@ int default_fused_planes(const DevParams& P, int halves)
     return planes;
 }
 
+// z chunk length of kz_scalars without lb_tune, by the same kind of model: 456
+// blocks at a time and five planes' time to start a block in FP32, the planes
+// of an SM's blocks in FP64.  Measured on GB300 (us, choice in brackets): FP32
+// 24^3 1 plane 13, 6 planes 21 [1]; 64^3 2 planes 14.7, 4 13.1, 16 17.1 [4];
+// 128^3 4 planes 56, 8 52, 12 50, 24 61 [8]; 256^3 8 planes 277, 24 250, 32 261,
+// 64 278 [32]; FP64 32^3 1 plane 63, 6 planes 140 [1]; 96^3 8 planes 428, 12
+// 406, 24 413 [12].
+int default_scalar_planes(const DevParams& P, bool fp64)
+{
+    const long long cols = (long long)((P.nx + 31) / 32) * ((P.ny + 7) / 8);
+    double best = 1e300;
+    int planes = 1;
+    for (int p = 1; p <= 64 && p <= P.nz; ++p) {
+        const int chunks = (P.nz + p - 1) / p;
+        if ((P.nz + chunks - 1) / chunks != p) continue;   // not the length of equal chunks
+        const long long blocks = cols * chunks;
+        const double cost = fp64 ? ((double)((blocks + 151) / 152) + 0.3) * (p + 1.3)
+                                 : (std::max(0.5, (double)blocks / 456) + 1.0) * (p + 5);
+        if (cost < best) {
+            best = cost;
+            planes = p;
+        }
+    }
+    return planes;
+}
+
 // Grid of a z-marching kernel with chunks of `planes` planes (no empty chunk).
 dim3 zm_grid(const DevParams& P, int planes)
 {
@@ -207,10 +218,10 @@ dim3 zm_grid(const DevParams& P, int planes)
 RowGrid row_grid(const lb_handle* h)
 {
     RowGrid g;
-    const int d = default_planes(h->dp);
-    const int halves = h->prm.precision == LB_FP64 ? 1 : 2;
-    g.zgrid = zm_grid(h->dp, h->zplanes[0] > 0 ? h->zplanes[0] : default_fused_planes(h->dp, halves));
-    g.zgrid_s = zm_grid(h->dp, h->zplanes[1] > 0 ? h->zplanes[1] : d);
+    const bool fp64 = h->prm.precision == LB_FP64;
+    const int* z = h->zplanes;
+    g.zgrid = zm_grid(h->dp, z[0] > 0 ? z[0] : default_fused_planes(h->dp, fp64 ? 1 : 2));
+    g.zgrid_s = zm_grid(h->dp, z[1] > 0 ? z[1] : default_scalar_planes(h->dp, fp64));
     return g;
 }
 

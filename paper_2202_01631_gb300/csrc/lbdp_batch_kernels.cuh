@@ -86,9 +86,9 @@ __global__ void __launch_bounds__(kZThreads, fused_blocks_per_sm<C>()) kbz_fused
 }
 
 template <class C, int ZC>
-__global__ void __launch_bounds__(kZThreads, kScalBlocksPerSM) kbz_scalars(const __grid_constant__ BoxLaunch L)
+__global__ void __launch_bounds__(kZThreads, scal_blocks_per_sm<C>()) kbz_scalars(const __grid_constant__ BoxLaunch L)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];   // sizeof(ScalSmem<F>)
+    extern __shared__ __align__(16) unsigned char smem_raw[];   // scal_smem_bytes<C>()
     const int b = blockIdx.y;
     if (b >= L.nbox || L.left[L.base + b] <= 0) return;
     const DevParams& P = L.box[b].P;

@@ -848,7 +848,7 @@ __device__ __forceinline__ void bulk_wall_links(const DevParams& P, const DevPtr
 // one packed instruction (each lane rounds as the scalar operation does);
 // FP64 keeps two scalar operations.
 template <class R>
-struct Two {
+struct alignas(2 * sizeof(R)) Two {
     R a, b;
 };
 __device__ __forceinline__ Two<float> fma2(Two<float> x, Two<float> y, Two<float> z)
@@ -866,6 +866,19 @@ __device__ __forceinline__ Two<float> add2(Two<float> x, Two<float> y)
     return {r.x, r.y};
 }
 __device__ __forceinline__ Two<double> add2(Two<double> x, Two<double> y) { return {add_x(x.a, y.a), add_x(x.b, y.b)}; }
+__device__ __forceinline__ Two<double> sub2(Two<double> x, Two<double> y)
+{
+    return {add_x(x.a, -y.a), add_x(x.b, -y.b)};
+}
+__device__ __forceinline__ Two<float> sub2(Two<float> x, Two<float> y)
+{
+    Two<float> r;
+    asm("{.reg .b64 a, b, c;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n sub.rn.f32x2 c, a, b;\n"
+        " mov.b64 {%0, %1}, c;}"
+        : "=f"(r.a), "=f"(r.b)
+        : "f"(x.a), "f"(x.b), "f"(y.a), "f"(y.b));
+    return r;
+}
 
 // Lattice-Boltzmann transport (scalar_scheme 1): D3Q7, weights 1/4 (rest)
 // and 1/8, c_s^2 = 1/4, relaxation time 1, Gamma = 2M.  The post-collision

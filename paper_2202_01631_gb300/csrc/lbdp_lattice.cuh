@@ -5,7 +5,8 @@
 //   populations  f[2][19][N]   storage type of the precision mode, pull scheme,
 //                              double buffered (read f[cur], write f[cur^1]);
 //   psi, phi     [2][N]        field type, double buffered;
-//   mu_psi, mu_phi, u[3]       [N] each, field type;
+//   mu_psi, mu_phi             [N][2], field type (as two [N] in a readout);
+//   u[3]                       [N] each, field type;
 //   mask         [2][N] u8     0 fluid, k+1 inside particle k, double buffered;
 //   particles    DevPart[np]   FP64 state.
 // Node index n = x + nx*(y + ny*z): x is the fastest axis, so a warp reads
@@ -211,8 +212,9 @@ struct DevPtrs {
     void* psi_dst;
     const void* phi_src;
     void* phi_dst;
-    void* mupsi;
+    void* mupsi;          // [N], [N]: the readout's chemical potentials (lb_read_mu) ...
     void* muphi;
+    void* mu;             // ... and in the same memory [N][2], the step's mu_psi, mu_phi
     void* pt;             // [kPtFields][N] chemical stress: p_iso (less A/4), grad psi
     void* force;          // [3][N] force on the fluid, g - div P
     void* u;

@@ -69,7 +69,7 @@ struct Ops {
     using F = typename C::fld_t;
 
     static constexpr size_t kFusedSmem = fused_smem_bytes<C>();
-    static constexpr size_t kZScalSmem = sizeof(ScalSmem<F>);
+    static constexpr size_t kZScalSmem = scal_smem_bytes<C>();
 
     // Opt the kernels that use more than 48 KiB of shared memory in, once per
     // device.
@@ -254,7 +254,7 @@ struct BOps {
         }
     }
 
-    static size_t smem(int nc) { return nc == 0 ? fused_smem_bytes<C>() : sizeof(ScalSmem<F>); }
+    static size_t smem(int nc) { return nc == 0 ? fused_smem_bytes<C>() : scal_smem_bytes<C>(); }
 
     static cudaError_t prepare()
     {

@@ -773,13 +773,28 @@ __global__ void __launch_bounds__(kPartThreads, part_blocks_per_sm<C>()) k_colli
 // ---------------------------------------------------------------------------
 // S4 next to particles, beside kz_scalars (which leaves those nodes out)
 // ---------------------------------------------------------------------------
+// Accessor of the transport body (scalars_compute_c) over global memory.
+template <class F>
+struct SAcc {
+    int nb[19];
+    int n, N;
+    const uint8_t* mk;
+    const F *psi, *phi, *mu, *u;
+    __device__ __forceinline__ uint8_t mask(int i) const { return nb[i] >= 0 ? mk[nb[i]] : kWallSlot; }
+    template <int K>
+    __device__ __forceinline__ F get(int i) const
+    {
+        const int m = nb[i] >= 0 ? nb[i] : n;
+        return K == 0 ? psi[m] : K == 1 ? phi[m] : K < 4 ? mu[2 * m + (K - 2)] : u[(K - 4) * N + m];
+    }
+};
+
 template <class C>
 __device__ __forceinline__ void scalars_particles_block(const DevParams& P, const DevPtrs& D, int p, int bi, int nbi,
                                                         NodeList& list)
 {
     using R = typename C::real;
     using F = typename C::fld_t;
-    const size_t N = (size_t)P.N;
     int o[3];
     link_box(D.parts[p], o);
     const int tot = P.side1[0] * P.side1[1] * P.side1[2];
@@ -793,27 +808,25 @@ __device__ __forceinline__ void scalars_particles_block(const DevParams& P, cons
         Around a;
         look_around(P, D, x, y, z, a);
         if (a.lo != p + 1) continue;
-        GAcc<F, 7> g;
+        SAcc<F> g;
 #pragma unroll
         for (int i = 0; i < 19; ++i) g.nb[i] = a.nb[i];
         g.n = n;
         g.mk = D.mask;
-        g.f[0] = (const F*)D.psi_src;
-        g.f[1] = (const F*)D.phi_src;
-        g.f[2] = (const F*)D.mupsi;
-        g.f[3] = (const F*)D.muphi;
-        g.f[4] = (const F*)D.u;
-        g.f[5] = (const F*)D.u + N;
-        g.f[6] = (const F*)D.u + 2 * N;
+        g.psi = (const F*)D.psi_src;
+        g.phi = (const F*)D.phi_src;
+        g.mu = (const F*)D.mu;
+        g.u = (const F*)D.u;
+        g.N = (int)P.N;
         const R dps = corr_r<R>(D, 0), dph = corr_r<R>(D, 1);
-        const R ps = (R)g.f[0][n] + dps, ph = (R)g.f[1][n] + dph;
+        const R ps = (R)g.psi[n] + dps, ph = (R)g.phi[n] + dph;
         // links into particles: no diffusive flux; the scalars leave with the
         // boundary velocity of the bounce-back rule, c.u_b g(x) -- weighted
         // w_i on the D3Q19 links of the finite-difference scheme, 1 on the six
         // D3Q7 links of the lattice-Boltzmann one; Janus production on the
         // m.(x - X) <= 0 side of each adjacent particle (any of the 18)
         R gphi[3];
-        grad_phi_around<R, F>(a, g.f[1], n, ph, dph, gphi);
+        grad_phi_around<R, F>(a, g.phi, n, ph, dph, gphi);
         R out = 0, src = 0;   // sum of w c.u_b
         for (int k = a.lo; k <= a.hi; ++k) {
             unsigned b = links_into(a, k);

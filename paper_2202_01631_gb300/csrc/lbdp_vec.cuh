@@ -82,6 +82,43 @@ __device__ __forceinline__ Vec<float, 2> recip(Vec<float, 2> a)
     return vfma(r, e, r);
 }
 
+// min(a, 0) and max(a, 0), NaN kept.  FP64 decides on the high word: comparing
+// takes the FP64 pipe.
+__device__ __forceinline__ float min0(float a)
+{
+    float r;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(0.0f));
+    return r;
+}
+__device__ __forceinline__ float max0(float a)
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(0.0f));
+    return r;
+}
+__device__ __forceinline__ double min0(double a) { return (unsigned)__double2hiint(a) <= 0x7FF00000u ? 0.0 : a; }
+__device__ __forceinline__ double max0(double a)
+{
+    const unsigned h = (unsigned)__double2hiint(a);
+    return h >= 0x80000000u && h <= 0xFFF00000u ? 0.0 : a;
+}
+template <class R, int NP>
+__device__ __forceinline__ Vec<R, NP> vmin0(Vec<R, NP> a)
+{
+    Vec<R, NP> r;
+#pragma unroll
+    for (int h = 0; h < NP; ++h) r.set(h, min0(a.lane(h)));
+    return r;
+}
+template <class R, int NP>
+__device__ __forceinline__ Vec<R, NP> vmax0(Vec<R, NP> a)
+{
+    Vec<R, NP> r;
+#pragma unroll
+    for (int h = 0; h < NP; ++h) r.set(h, max0(a.lane(h)));
+    return r;
+}
+
 // a scalar factor or addend
 template <class R, int NP>
 __device__ __forceinline__ Vec<R, NP> operator*(R a, Vec<R, NP> b) { return Vec<R, NP>::of(a) * b; }

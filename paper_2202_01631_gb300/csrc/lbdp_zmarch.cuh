@@ -12,7 +12,7 @@
 //               side-stream kernels (k_pt_part, k_f_part,
 //               k_collide_particles).
 //   kz_scalars  the psi/phi transport (Eq. diffusion_reaction) from a ring of
-//               three 34 x 10 planes of psi, phi, mu and u.
+//               34 x 10 planes of psi, phi, mu and u.
 //
 // A tile column is one thread; a block walks ZC planes (its z chunk) with
 // one barrier per plane.  Halo planes of a chunk are staged (and, for the
@@ -39,26 +39,7 @@ __host__ __device__ constexpr int poff(int i)
     return cx(i) + W * cy(i);
 }
 
-// shape of a one-halo plane for the paired field layout (tile_index_last)
-struct ZPlane1 {
-    static constexpr int slots = kZ1;
-};
-
-// Shared-memory place of field k of slot s in a plane of T::slots slots:
-// fields 2j and 2j+1 interleave ([j][slot][2]), so a body that reads both
-// gets them in one 64-bit load; an odd last field stands alone.
-template <class T>
-__host__ __device__ constexpr int tile_index(int k, int s)
-{
-    return (k & ~1) * T::slots + 2 * s + (k & 1);
-}
-template <int NF, class T>
-__host__ __device__ constexpr int tile_index_last(int k, int s)
-{
-    return ((NF & 1) && k == NF - 1) ? (NF - 1) * T::slots + s : tile_index<T>(k, s);
-}
-
-// Nodes a thread of kz_fused works on together: the node of its column in each
+// Nodes a thread of a bulk kernel works on together: the node of its column in each
 // half of the block's z chunk.  Two in FP32 arithmetic (packed instructions,
 // one set of column offsets, 64-bit shared loads); one in FP64, which has no
 // packed form and no registers to spare.
@@ -69,16 +50,19 @@ __host__ __device__ constexpr int zm_halves()
 }
 
 // Particles whose nodes may lie in the columns a block stages: the planes lo
-// .. lo + len - 1 (before wrapping) hold them; slot[k] is where particle k
-// stands in the list.  geo: what the wetting ghosts need of it.
+// .. lo + len - 1 (before wrapping) hold them.
+struct SolidPlanes {
+    int n;
+    int lo[kMaxParticles], len[kMaxParticles];
+};
+// What the wetting ghosts of kz_fused need of them; slot[k] is where particle
+// k stands in the list.
 struct GhostPart {
     Geo g;
     double Hk;
     float Hk_f;
 };
-struct SolidPlanes {
-    int n;
-    int lo[kMaxParticles], len[kMaxParticles];
+struct GhostParts {
     uint8_t slot[kMaxParticles];
     GhostPart geo[kMaxParticles];
 };
@@ -93,6 +77,7 @@ struct FusedSmem {
     F psi[kPsiRing][kZ2][NP];
     F phi[kPhiRing][kZ1][NP];
     SolidPlanes sol;
+    GhostParts ghost;
     // nodes of the plane in hand that take the general body (NP slot + half),
     // and how many, for even and odd iterations
     uint16_t todo[NP * kZ1];
@@ -101,8 +86,10 @@ struct FusedSmem {
 
 template <class F>
 struct ScalSmem {
-    F f[kScalRing][7 * kZ1];
-    uint8_t mk[kScalRing][kZ1];
+    F g[kScalRing][kZ1][2];    // psi, phi
+    F mu[kScalRing][kZ1][2];   // mu_psi, mu_phi
+    F u[kScalRing][3][kZ1];
+    SolidPlanes sol;
 };
 
 // Column coordinate of halo offset l (may be negative) from tile origin o on
@@ -128,9 +115,12 @@ __device__ __forceinline__ bool spans_meet(int lo, int len, int o, int flen, int
 }
 
 // The particles near the block's columns (grown by halo on each side), at the
-// positions the current mask was made from.
+// positions the current mask was made from; extra(k, i, record) takes particle
+// k, i-th of the list.  kNew: from the positions after this step's particle
+// update (gn), grown by what a step's velocity moves them.
+template <bool kNew, class Fn>
 __device__ __forceinline__ void find_solids(const DevParams& P, const DevPtrs& D, int x0, int y0, int halo,
-                                            SolidPlanes& sp)
+                                            SolidPlanes& sp, Fn extra)
 {
     if (threadIdx.x == 0) sp.n = 0;
     __syncthreads();
@@ -138,16 +128,19 @@ __device__ __forceinline__ void find_solids(const DevParams& P, const DevPtrs& D
         const DevPart& q = D.parts[k];
         // |x - X| < R lies strictly between floor(X) - ceil(R) and
         // floor(X) + ceil(R) + 1
-        const int w = 2 * q.Rc + 2;
-        if (spans_meet(q.g.Xi[0] - q.Rc, w, x0 - halo, kZX + 2 * halo, P.nx, P.per[0]) &&
-            spans_meet(q.g.Xi[1] - q.Rc, w, y0 - halo, kZY + 2 * halo, P.ny, P.per[1])) {
+        int lo[3], w[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const int g = kNew ? 1 + (int)ceilf(fabsf(q.Uf[a])) : 0;
+            lo[a] = (kNew ? q.gn.Xi[a] : q.g.Xi[a]) - q.Rc - g;
+            w[a] = 2 * (q.Rc + 1 + g);
+        }
+        if (spans_meet(lo[0], w[0], x0 - halo, kZX + 2 * halo, P.nx, P.per[0]) &&
+            spans_meet(lo[1], w[1], y0 - halo, kZY + 2 * halo, P.ny, P.per[1])) {
             const int i = atomicAdd(&sp.n, 1);
-            sp.lo[i] = q.g.Xi[2] - q.Rc;
-            sp.len[i] = w;
-            sp.slot[k] = (uint8_t)i;
-            sp.geo[i].g = q.g;
-            sp.geo[i].Hk = q.Hk;
-            sp.geo[i].Hk_f = q.Hk_f;
+            sp.lo[i] = lo[2];
+            sp.len[i] = w[2];
+            extra(k, i, q);
         }
     }
     __syncthreads();
@@ -180,8 +173,8 @@ struct ZAccMu {
     const F* ps[3];
     int o2;   // NP * slot + half
     F phi_own;
-    const SolidPlanes* sol;
-    __device__ __forceinline__ const GhostPart& part(const DevPtrs&, int k) const { return sol->geo[sol->slot[k]]; }
+    const GhostParts* gp;
+    __device__ __forceinline__ const GhostPart& part(const DevPtrs&, int k) const { return gp->geo[gp->slot[k]]; }
     __device__ __forceinline__ uint8_t mask(int i) const { return nb[i] >= 0 ? mk[nb[i]] : kWallSlot; }
     template <int K>
     __device__ __forceinline__ F get(int i) const
@@ -191,21 +184,24 @@ struct ZAccMu {
     }
 };
 
+// Bit 2 a + s of beyond: the neighbours on side s (0 below, 1 above) of axis a
+// lie beyond a wall.
+__device__ __forceinline__ bool beyond_wall(unsigned beyond, int i)
+{
+    const unsigned c = (cx(i) < 0 ? 1u : cx(i) > 0 ? 2u : 0u) | (cy(i) < 0 ? 4u : cy(i) > 0 ? 8u : 0u) |
+                       (cz(i) < 0 ? 16u : cz(i) > 0 ? 32u : 0u);
+    return (beyond & c) != 0;
+}
+
 // force body of a node next to a wall, in one half of the planes of kz_fused:
-// the stress (p_iso, grad psi) of the one-halo planes.  Bit 2 a + s of beyond:
-// the neighbours on side s (0 below, 1 above) of axis a lie beyond a wall.
+// the stress (p_iso, grad psi) of the one-halo planes
 template <class F, int NP>
 struct ZAccP {
     const F* pa[3];
     const F* pb[3];
     int o1;   // 2 * NP * slot + half
     unsigned beyond;
-    __device__ __forceinline__ uint8_t mask(int i) const
-    {
-        const unsigned c = (cx(i) < 0 ? 1u : cx(i) > 0 ? 2u : 0u) | (cy(i) < 0 ? 4u : cy(i) > 0 ? 8u : 0u) |
-                           (cz(i) < 0 ? 16u : cz(i) > 0 ? 32u : 0u);
-        return (beyond & c) ? kWallSlot : (uint8_t)0;
-    }
+    __device__ __forceinline__ uint8_t mask(int i) const { return beyond_wall(beyond, i) ? kWallSlot : (uint8_t)0; }
     template <int K>
     __device__ __forceinline__ F get(int i) const
     {
@@ -214,20 +210,21 @@ struct ZAccP {
     }
 };
 
-// transport body: psi, phi, mu_psi, mu_phi, u (one-halo planes, paired)
-template <class F, bool kClear>
+// transport body of a node next to a wall: psi, phi, mu_psi, mu_phi, u of the
+// one-halo planes of kz_scalars
+template <class F>
 struct ZAccS {
-    const F* f[3];
-    const uint8_t* mk[3];
+    const F (*g[3])[2];
+    const F (*mu[3])[2];
+    const F (*u[3])[kZ1];
     int s1;
-    __device__ __forceinline__ uint8_t mask(int i) const
-    {
-        return kClear ? (uint8_t)0 : mk[1 + cz(i)][s1 + poff<kZ1X>(i)];
-    }
+    unsigned beyond;
+    __device__ __forceinline__ uint8_t mask(int i) const { return beyond_wall(beyond, i) ? kWallSlot : (uint8_t)0; }
     template <int K>
     __device__ __forceinline__ F get(int i) const
     {
-        return f[1 + cz(i)][tile_index_last<7, ZPlane1>(K, s1 + poff<kZ1X>(i))];
+        const int p = 1 + cz(i), s = s1 + poff<kZ1X>(i);
+        return K < 2 ? g[p][s][K] : K < 4 ? mu[p][s][K - 2] : u[p][K < 4 ? 0 : K - 4][s];
     }
 };
 
@@ -239,7 +236,7 @@ struct ZAccS {
 template <int B>
 __device__ __forceinline__ void cp_async(void* sdst, const void* gsrc, bool valid)
 {
-    static_assert(B == 4 || B == 8, "4- or 8-byte copies");
+    static_assert(B == 4 || B == 8 || B == 16, "4-, 8- or 16-byte copies");
     const unsigned s = (unsigned)__cvta_generic_to_shared(sdst);
     // src-size 0 writes zeros and reads nothing (a slot beyond a wall)
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;\n" ::"r"(s), "l"(gsrc), "n"(B),
@@ -346,61 +343,6 @@ __device__ __forceinline__ void scal_cols(const DevParams& P, int x0, int y0, Sc
             if (gx >= 0 && gy >= 0) c.c[h] = gx + P.nx * gy;
         }
     }
-}
-
-// Issue the copies of the seven transport fields of plane p into ring slot r.
-template <class F>
-__device__ __forceinline__ void scal_plane_async(const DevParams& P, const DevPtrs& D, const ScalCols& c, int p,
-                                                 ScalSmem<F>& sm, int r)
-{
-    const size_t N = (size_t)P.N;
-    const F* u = (const F*)D.u;
-    const F* const src[7] = {(const F*)D.psi_src, (const F*)D.phi_src, (const F*)D.mupsi, (const F*)D.muphi,
-                             u, u + N, u + 2 * N};
-    const int gz = wrap_coord(p, P.nz, P.per[2]);
-    const int base = gz * P.nx * P.ny;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int s = threadIdx.x + h * kZThreads;
-        if (s < kZ1) {
-            const bool ok = c.c[h] >= 0 && gz >= 0;
-            const int g = ok ? base + c.c[h] : 0;
-#pragma unroll
-            for (int k = 0; k < 7; ++k)
-                cp_async<(int)sizeof(F)>(&sm.f[r][tile_index_last<7, ZPlane1>(k, s)], src[k] + g, ok);
-        }
-    }
-}
-
-// The masks of a plane go through registers (their OR decides the mask-free
-// body): m[h] for this thread's slots, kWallSlot beyond a wall.
-struct ScalMask {
-    uint8_t m[2];
-};
-
-__device__ __forceinline__ void scal_mask_fetch(const DevParams& P, const DevPtrs& D, const ScalCols& c, int p,
-                                                ScalMask& M)
-{
-    const int gz = wrap_coord(p, P.nz, P.per[2]);
-    const int base = gz * P.nx * P.ny;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) M.m[h] = (c.c[h] >= 0 && gz >= 0) ? D.mask[base + c.c[h]] : kWallSlot;
-}
-
-// Store the masks into ring slot r; returns whether any is not fluid.
-template <class F>
-__device__ __forceinline__ bool scal_mask_store(ScalSmem<F>& sm, int r, const ScalMask& M)
-{
-    bool any = false;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int s = threadIdx.x + h * kZThreads;
-        if (s < kZ1) {
-            sm.mk[r][s] = M.m[h];
-            any = any || M.m[h] != 0;
-        }
-    }
-    return any;
 }
 
 // Planes per z chunk of a launch with gridDim.z chunks.
@@ -513,10 +455,7 @@ __device__ __forceinline__ void mu_put(const DevPtrs& D, FusedSmem<F, NP>& sm, b
         sm.pb[rt][q][h] = (F)pt[2];
         sm.pb[rt][q][NP + h] = (F)pt[3];
     }
-    if (n >= 0) {
-        ((F*)D.mupsi)[n] = (F)mps;
-        ((F*)D.muphi)[n] = (F)mph;
-    }
+    if (n >= 0) ((Two<F>*)D.mu)[n] = {(F)mps, (F)mph};
 }
 
 // Stage 1 of one plane per half (zs): mu and the stress of the 34 x 10
@@ -575,8 +514,7 @@ __device__ __forceinline__ void fused_stage1(const DevParams& P, const DevPtrs& 
             for (int h = 0; h < NP; ++h)
                 if (own[h] && (kQuiet || !(skip >> h & 1u))) {
                     const int n = wcol + sxy * zs[h];
-                    ((F*)D.mupsi)[n] = (F)mps.lane(h);
-                    ((F*)D.muphi)[n] = (F)mph.lane(h);
+                    ((Two<F>*)D.mu)[n] = {(F)mps.lane(h), (F)mph.lane(h)};
                 }
         }
     }
@@ -597,7 +535,7 @@ __device__ __forceinline__ void fused_stage1(const DevParams& P, const DevPtrs& 
         for (int j = 0; j < 3; ++j) a.ps[j] = &sm.psi[rp[j]][0][0];
         a.o2 = NP * ((lx + 2) + kZ2X * (ly + 2)) + h;
         a.phi_own = sm.phi[rf][q][h];
-        a.sol = &sm.sol;
+        a.gp = &sm.ghost;
         R m1, m2, p4[kPtFields];
         mup_values<C>(P, D, x, y, z, a, dps.lane(0), dph.lane(0), m1, m2, p4);
         const bool put = (h == 0 ? own[0] : own[NP - 1]) && lx >= 0 && lx < kZX && ly >= 0 && ly < kZY &&
@@ -992,7 +930,12 @@ __device__ __forceinline__ void kz_fused_run(const DevParams& P, const DevPtrs& 
     constexpr int NP = zm_halves<R>();
     static_assert(sizeof(R) == sizeof(F), "the staged planes are read as arithmetic vectors");
     FusedSmem<F, NP>& sm = *reinterpret_cast<FusedSmem<F, NP>*>(smem_raw);
-    find_solids(P, D, x0, y0, 2, sm.sol);
+    find_solids<false>(P, D, x0, y0, 2, sm.sol, [&](int k, int i, const DevPart& q) {
+        sm.ghost.slot[k] = (uint8_t)i;
+        sm.ghost.geo[i].g = q.g;
+        sm.ghost.geo[i].Hk = q.Hk;
+        sm.ghost.geo[i].Hk_f = q.Hk_f;
+    });
     const bool xywall = beyond_xy(P, x0, y0, 2);
     // planes any iteration looks at: z0 - 2 .. z0 + NP na + 1
     bool quiet = !xywall && (P.per[2] || (z0 >= 2 && z0 + nt + NP + 1 <= P.nz));
@@ -1026,85 +969,375 @@ __global__ void __launch_bounds__(kZThreads, fused_blocks_per_sm<C>()) kz_fused(
 // ---------------------------------------------------------------------------
 // kz_scalars
 // ---------------------------------------------------------------------------
-template <class C, bool kClear>
-__device__ __forceinline__ void scal_stage(const DevParams& P, const DevPtrs& D,
-                                           const ScalSmem<typename C::fld_t>& sm, int x0, int y0, int zs,
-                                           const int (&r)[3], typename C::real dps, typename C::real dph)
+// What bounds the transport is instruction issue and shared-memory bandwidth
+// (18 neighbours of seven fields per node), so:
+//   - the links are taken plane by plane: when plane q arrives, its eight
+//     neighbours of a column are read once and serve the in-plane links of
+//     plane q and the links up to it from q - 1 and down to it from q + 1
+//     (ScalSums), half the reads of 18 neighbours per node;
+//   - the linear parts, M lap mu and the divergence of u, are sums over a plane
+//     that the three planes share; the upwind part is left with one minimum
+//     and two multiply-adds per link:
+//       sum_i w_i [M (mu_i - mu) - (ub g)_upwind],  b_i = c.(u + u_i) = 2 ub_i,
+//       = sum_i w_i [M (mu_i - mu) - (min(b_i, 0) (g_i - g) + c.u_i g) / 2]
+//     (sum_i w_i c.u = 0);
+//   - the sink k_d (phi - phi0) is (k_d / C) mu_phi, which is staged already;
+//   - psi and phi, and mu_psi and mu_phi, lie side by side in shared memory and
+//     go through packed FP32 instructions.
+// Solid nodes and those next to particles are left out, nodes next to walls
+// take the general body; which form a node takes depends on the node alone.
+// One node per thread and 24 warps per SM: with two nodes per thread, as in
+// kz_fused, the kernel issues a fifth fewer instructions but has 16 warps and
+// waits more.  Measured on GB300, eight spheres at 256^3, FP32: 344 us with 18
+// neighbours per node, 328 with two nodes per thread, 250 so; FP64 96^3 549 ->
+// 406 us, there by the FP64 operations saved.
+
+// Issue the copies of the seven transport fields of plane p into ring slot r.
+template <class F, bool kQuiet>
+__device__ __forceinline__ void scal_plane_async(const DevParams& P, const DevPtrs& D, const ScalCols& c, int p,
+                                                 ScalSmem<F>& sm, int r)
 {
-    using F = typename C::fld_t;
-    const int tx = threadIdx.x & (kZX - 1), ty = threadIdx.x / kZX;
-    const int x = x0 + tx, y = y0 + ty;
-    if (x >= P.nx || y >= P.ny) return;
-    const int s1 = (tx + 1) + kZ1X * (ty + 1);
-    if (sm.mk[r[1]][s1] != 0) return;   // inside a particle
-    ZAccS<F, kClear> a;
+    const int NN = (int)P.N;
+    const F* psi = (const F*)D.psi_src;
+    const F* phi = (const F*)D.phi_src;
+    const F* mu = (const F*)D.mu;
+    const F* u = (const F*)D.u;
+    const int gz = wrap_coord(p, P.nz, P.per[2]);
+    const int base = !kQuiet && gz < 0 ? 0 : gz * P.nx * P.ny;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        a.f[k] = sm.f[r[k]];
-        a.mk[k] = sm.mk[r[k]];
+    for (int k = 0; k < 2; ++k) {
+        const int s = threadIdx.x + k * kZThreads;
+        if (k == 0 || s < kZ1) {
+            const bool ok = kQuiet || (c.c[k] >= 0 && gz >= 0);
+            const int g = ok ? base + c.c[k] : 0;
+            cp_async<(int)sizeof(F)>(&sm.g[r][s][0], psi + g, ok);
+            cp_async<(int)sizeof(F)>(&sm.g[r][s][1], phi + g, ok);
+            cp_async<2 * (int)sizeof(F)>(&sm.mu[r][s][0], mu + 2 * g, ok);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) cp_async<(int)sizeof(F)>(&sm.u[r][a][s], u + (a * NN + g), ok);
+        }
     }
-    a.s1 = s1;
-    scalars_compute_c<C, false>(P, D, x, y, zs, x + P.nx * (y + P.ny * zs), a, dps, dph);
 }
 
-// The march of one block, as kz_fused_run (smem of sizeof(ScalSmem<F>) bytes).
-template <class C>
-__device__ __forceinline__ void kz_scalars_run(const DevParams& P, const DevPtrs& D, int x0, int y0, int z0, int nt,
-                                               unsigned char* smem_raw)
+// The sums of one node over the planes seen so far, in units of the diagonal
+// weight 1/36 (axis links count twice): ad = sum min(b, 0) (g_i - g) for psi
+// and phi, dv = sum c.u_i, lp = sum (mu_i - mu) for both.
+template <class R>
+struct ScalSums {
+    Two<R> ad, lp;
+    R dv;
+};
+
+// A column's own psi, phi and u in one plane.
+template <class R>
+struct ScalOwn {
+    Two<R> g;
+    R u[3];
+};
+
+// One plane of the ring.
+template <class R>
+struct ScalPlane {
+    const R (*g)[2];
+    const R (*mu)[2];
+    const R (*u)[kZ1];
+    __device__ __forceinline__ Two<R> gp(int s) const { return *reinterpret_cast<const Two<R>*>(g[s]); }
+    __device__ __forceinline__ Two<R> mp(int s) const { return *reinterpret_cast<const Two<R>*>(mu[s]); }
+};
+template <class F>
+__device__ __forceinline__ ScalPlane<F> scal_ring(const ScalSmem<F>& sm, int r)
+{
+    return {sm.g[r], sm.mu[r], sm.u[r]};
+}
+
+template <class R>
+__device__ __forceinline__ ScalOwn<R> scal_own(const ScalPlane<R>& f, int s)
+{
+    return {f.gp(s), {f.u[0][s], f.u[1][s], f.u[2][s]}};
+}
+
+// One link: b = c.(u + u_i) (minus it when kNeg) and the difference d of psi
+// and phi along it, into the upwind sums.
+template <bool kNeg, class R>
+__device__ __forceinline__ void upwind(R b, Two<R> d, Two<R>& a)
+{
+    const R m = kNeg ? -max0(b) : min0(b);   // min(-b, 0) = -max(b, 0)
+    a.a = fma_x(m, d.a, a.a);
+    a.b = fma_x(m, d.b, a.b);
+}
+
+// Take in plane q (f): completes prev, the sums of the node below, adds the
+// in-plane links to cur and starts next, the node above.  a, o, b: the
+// column's own values in planes q - 1, q, q + 1; mm, m0: mu_psi, mu_phi of the
+// column in planes q - 1 and q.  inner: the node of plane q is of this chunk.
+template <class R>
+__device__ __forceinline__ void scal_plane(const ScalPlane<R>& f, int s1, bool inner, const ScalOwn<R>& a,
+                                           const ScalOwn<R>& o, const ScalOwn<R>& b, Two<R> mm, Two<R> m0,
+                                           ScalSums<R>& prev, ScalSums<R>& cur, ScalSums<R>& next)
+{
+    constexpr int Y = kZ1X;
+    // the column itself: links up from q - 1 and down from q + 1
+    {
+        const R bu = add_x(a.u[2], o.u[2]), bd = add_x(b.u[2], o.u[2]);
+        next.ad = {0, 0};
+        upwind<false>(add_x(bu, bu), sub2(o.g, a.g), prev.ad);
+        upwind<true>(add_x(bd, bd), sub2(o.g, b.g), next.ad);
+    }
+    R e = 0, z4 = 0;             // in-plane sums over the axis neighbours
+    Two<R> l4{0, 0}, ad2{0, 0};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {   // +x, -x, +y, -y
+        const int ax = k / 2;
+        const bool neg = k & 1;
+        const int s = s1 + (neg ? -1 : 1) * (ax == 0 ? 1 : Y);
+        const Two<R> g = f.gp(s);
+        const R nu = f.u[ax][s], nz = f.u[2][s];
+        l4 = add2(l4, sub2(f.mp(s), m0));
+        z4 = add_x(z4, nz);
+        e = neg ? add_x(e, -nu) : add_x(e, nu);
+        const R bi = add_x(o.u[ax], nu);   // c.(u + u_i) in the plane, minus it on the negative side
+        // c = (+-1, 0, 1) from q - 1: +-(u + u_i) + (uz + uz_i); (+-1, 0, -1) from q + 1
+        const R az = add_x(a.u[2], nz), an = add_x(a.u[ax], nu), bz = add_x(b.u[2], nz), bn = add_x(b.u[ax], nu);
+        if (neg) {
+            upwind<true>(bi, sub2(g, o.g), ad2);
+            upwind<false>(add_x(az, -an), sub2(g, a.g), prev.ad);
+            upwind<true>(add_x(bz, bn), sub2(g, b.g), next.ad);
+        } else {
+            upwind<false>(bi, sub2(g, o.g), ad2);
+            upwind<false>(add_x(az, an), sub2(g, a.g), prev.ad);
+            upwind<true>(add_x(bz, -bn), sub2(g, b.g), next.ad);
+        }
+    }
+    const R Z = fma_x((R)2, o.u[2], z4);
+    const Two<R> d6 = sub2(m0, mm);
+    prev.dv = add_x(prev.dv, add_x(e, Z));
+    prev.lp = add2(prev.lp, fma2(Two<R>{6, 6}, d6, l4));
+    next.dv = add_x(e, -Z);
+    next.lp = l4;
+    if (!inner) return;
+    // diagonal neighbours in the plane
+    const R us = add_x(o.u[0], o.u[1]), ud = add_x(o.u[0], -o.u[1]);
+    R v = 0;
+    Two<R> d4{0, 0};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {   // (1,1), (-1,-1), (1,-1), (-1,1)
+        const bool neg = k & 1, anti = k >= 2;
+        const int s = s1 + (neg ? -1 : 1) * (anti ? 1 - Y : 1 + Y);
+        const Two<R> g = f.gp(s);
+        const R nx = f.u[0][s], ny = f.u[1][s];
+        d4 = add2(d4, sub2(f.mp(s), m0));
+        const R cu = anti ? add_x(nx, -ny) : add_x(nx, ny);
+        v = neg ? add_x(v, -cu) : add_x(v, cu);
+        const R bi = add_x(anti ? ud : us, cu);
+        if (neg)
+            upwind<true>(bi, sub2(g, o.g), cur.ad);
+        else
+            upwind<false>(bi, sub2(g, o.g), cur.ad);
+    }
+    cur.ad = fma2(Two<R>{2, 2}, ad2, cur.ad);
+    cur.dv = add_x(cur.dv, fma_x((R)2, e, v));
+    cur.lp = add2(cur.lp, fma2(Two<R>{-6, -6}, d6, fma2(Two<R>{2, 2}, l4, d4)));
+}
+
+// The lattice-Boltzmann transport of a clear node (scalars_compute_lb) from
+// the planes below, own and above: the increments of psi and phi less the
+// correction and the sink.
+template <class R>
+__device__ __forceinline__ Two<R> scal_lb(const PrmR<R>& Q, const ScalPlane<R>& f0, const ScalPlane<R>& f1,
+                                          const ScalPlane<R>& f2, int s1, Two<R> corr)
+{
+    const Two<R> m0 = f1.mp(s1);
+    Two<R> l{0, 0}, ad{0, 0};
+#pragma unroll
+    for (int i = 1; i < 7; ++i) {
+        const ScalPlane<R>& f = cz(i) == 0 ? f1 : cz(i) > 0 ? f2 : f0;
+        const int s = s1 + poff<kZ1X>(i), a = cx(i) != 0 ? 0 : cy(i) != 0 ? 1 : 2;
+        const R u = cx(i) + cy(i) + cz(i) < 0 ? -f.u[a][s] : f.u[a][s];
+        const Two<R> g = add2(f.gp(s), corr);
+        l = add2(l, sub2(f.mp(s), m0));
+        ad.a = fma_x(u, g.a, ad.a);
+        ad.b = fma_x(u, g.b, ad.b);
+    }
+    return {fma_x((R)-0.5, ad.a, mul_x(Q.Mpsi, l.a)), fma_x((R)-0.5, ad.b, mul_x(Q.Mphi, l.b))};
+}
+
+// Whether (x, y, z) is fluid and not next to a particle, from the masks of this
+// step: covering replaces the boundary flags while this kernel runs.
+__device__ __forceinline__ bool free_node(const DevParams& P, const DevPtrs& D, int x, int y, int z)
+{
+    int nb[19];
+    neighbours(P, x, y, z, nb);
+    unsigned any = 0;
+#pragma unroll
+    for (int i = 0; i < 19; ++i) any |= D.mask[nb[i] >= 0 ? nb[i] : nb[0]];
+    return any == 0;
+}
+
+// The march of one block: columns x0 .. x0 + 31, y0 .. y0 + 7, planes z0 ..
+// z0 + nt - 1 (nt >= 1).  kQuiet: every plane the block stages is clear.  kLB:
+// the lattice-Boltzmann scheme.
+template <class C, bool kQuiet, bool kLB>
+__device__ __forceinline__ void scal_march(const DevParams& P, const DevPtrs& D, int x0, int y0, int z0, int nt,
+                                           bool xywall, ScalSmem<typename C::fld_t>& sm)
 {
     using R = typename C::real;
     using F = typename C::fld_t;
-    ScalSmem<F>& sm = *reinterpret_cast<ScalSmem<F>*>(smem_raw);
+    const PrmR<R>& Q = prm<R>(P);
     ScalCols cols;
     scal_cols(P, x0, y0, cols);
-    const R dps = corr_r<R>(D, 0), dph = corr_r<R>(D, 1);
-    // Plane p in ring slot (p - z0 + 1) mod 5.  Iteration t computes plane
-    // z0 + t from planes z0 + t - 1 .. z0 + t + 1 and issues the copies of
-    // plane z0 + t + 2 (into the slot of z0 + t - 3, last read at t - 2); the
-    // masks of a plane are loaded one iteration before they are stored.
-    unsigned hist = 0;
-    ScalMask M;
-    for (int k = 0; k < 2; ++k) {   // planes z0 - 1, z0
-        scal_plane_async<F>(P, D, cols, z0 - 1 + k, sm, k);
-        scal_mask_fetch(P, D, cols, z0 - 1 + k, M);
-        hist = (hist << 1) | (unsigned)__syncthreads_or(scal_mask_store<F>(sm, k, M));
-    }
+    const int tx = threadIdx.x & (kZX - 1), ty = threadIdx.x / kZX;
+    const int s1 = (tx + 1) + kZ1X * (ty + 1);
+    const int x = x0 + tx, y = y0 + ty;
+    const bool in = x < P.nx && y < P.ny;
+    const int nxy = x + P.nx * y, sxy = P.nx * P.ny;
+    const unsigned wxy = (!P.per[0] ? (x == 0 ? 1u : 0u) | (x == P.nx - 1 ? 2u : 0u) : 0u) |
+                         (!P.per[1] ? (y == 0 ? 4u : 0u) | (y == P.ny - 1 ? 8u : 0u) : 0u);
+    const Two<R> corr{corr_r<R>(D, 0), corr_r<R>(D, 1)};
+    const R kdc = Q.C != (R)0 ? Q.kd / Q.C : (R)0;
+    // Plane p in ring slot (p - z0 + 1) mod 5.  Iteration t takes in plane q =
+    // z0 + t - 1 (with the column's values in q + 1), finishes plane q - 1 and
+    // issues the copies of plane q + 2 into the slot of q - 3, last read in
+    // iteration t - 1.  Bit k of win: plane q + 1 - k is not clear.
+    unsigned win = 0;
+    if (!kQuiet)
+        win = ((unsigned)plane_solid(P, sm.sol, xywall, z0 - 2) << 1) |
+              (unsigned)plane_solid(P, sm.sol, xywall, z0 - 1);
+    scal_plane_async<F, kQuiet>(P, D, cols, z0 - 1, sm, 0);
+    scal_plane_async<F, kQuiet>(P, D, cols, z0, sm, 1);
     cp_async_commit();
-    scal_plane_async<F>(P, D, cols, z0 + 1, sm, 2);
-    cp_async_commit();
-    scal_mask_fetch(P, D, cols, z0 + 1, M);
-    int r0 = 0;   // slot of plane z0 + t - 1
-    for (int t = 0; t < nt; ++t) {
+    ScalSums<R> prev, cur, next;
+    ScalOwn<R> a, o;
+    Two<R> mm;
+    int r0 = 0;   // slot of plane q
+#pragma unroll 1
+    for (int t = 0; t <= nt + 1; ++t) {
         const int r1 = r0 + 1 == kScalRing ? 0 : r0 + 1;
         const int r2 = r1 + 1 == kScalRing ? 0 : r1 + 1;
-        const int r3 = r2 + 1 == kScalRing ? 0 : r2 + 1;
-        const bool any = scal_mask_store<F>(sm, r2, M);   // plane z0 + t + 1
-        if (t + 2 <= nt) {
-            scal_mask_fetch(P, D, cols, z0 + t + 2, M);
-            scal_plane_async<F>(P, D, cols, z0 + t + 2, sm, r3);
-        }
+        const int rm = r0 == 0 ? kScalRing - 1 : r0 - 1, rn = rm == 0 ? kScalRing - 1 : rm - 1;
+        cp_async_wait<0>();   // this thread's copies of plane q + 1 have landed
+        __syncthreads();
+        if (t + 1 <= nt) scal_plane_async<F, kQuiet>(P, D, cols, z0 + t + 1, sm, r2);   // plane q + 2
         cp_async_commit();
-        cp_async_wait<1>();   // this thread's copies of plane z0 + t + 1 have landed
-        hist = (hist << 1) | (unsigned)__syncthreads_or(any);
-        const int r[3] = {r0, r1, r2};
-        if ((hist & 7u) == 0u)
-            scal_stage<C, true>(P, D, sm, x0, y0, z0 + t, r, dps, dph);
-        else
-            scal_stage<C, false>(P, D, sm, x0, y0, z0 + t, r, dps, dph);
+        const int zo = z0 + t - 2;
+        bool put = in && t >= 2, wall = false;
+        if (!kQuiet) {
+            win = (win << 1) | (unsigned)plane_solid(P, sm.sol, xywall, z0 + t);
+            if (put && (win & 0xEu)) {   // planes q - 2 .. q
+                put = free_node(P, D, x, y, zo);
+                wall = wxy || (!P.per[2] && (zo == 0 || zo == P.nz - 1));
+            }
+        }
+        Two<R> inc, old;   // increments of psi, phi (less the correction and the sink), old values
+        R om;              // mu_phi
+        if (kLB) {
+            if (t >= 2) {
+                const ScalPlane<R> f1 = scal_ring(sm, rm);
+                inc = scal_lb<R>(Q, scal_ring(sm, rn), f1, scal_ring(sm, r0), s1, corr);
+                old = f1.gp(s1);
+                om = sm.mu[rm][s1][1];
+            }
+        } else {
+            const ScalPlane<R> f = scal_ring(sm, r0);
+            const Two<R> m0 = f.mp(s1);
+            if (t == 0) {
+                a = o = scal_own(f, s1);
+                mm = m0;
+                prev.ad = prev.lp = {0, 0};
+                prev.dv = 0;
+                cur = prev;
+            }
+            const ScalOwn<R> b = scal_own(scal_ring(sm, r1), s1);
+            scal_plane<R>(f, s1, t >= 1 && t <= nt, a, o, b, mm, m0, prev, cur, next);
+            old = a.g;
+            om = mm.b;
+            const Two<R> g = add2(old, corr);
+            inc.a = fma_x((R)(-1.0 / 12.0), fma_x(g.a, prev.dv, prev.ad.a), mul_x((R)(1.0 / 6.0) * Q.Mpsi, prev.lp.a));
+            inc.b = fma_x((R)(-1.0 / 12.0), fma_x(g.b, prev.dv, prev.ad.b), mul_x((R)(1.0 / 6.0) * Q.Mphi, prev.lp.b));
+            prev = cur;
+            cur = next;
+            a = o;
+            o = b;
+            mm = m0;
+        }
+        if (put) {
+            const int n = nxy + sxy * zo;
+            if (!kQuiet && wall) {
+                ZAccS<F> w;
+                w.g[0] = sm.g[rn];
+                w.g[1] = sm.g[rm];
+                w.g[2] = sm.g[r0];
+                w.mu[0] = sm.mu[rn];
+                w.mu[1] = sm.mu[rm];
+                w.mu[2] = sm.mu[r0];
+                w.u[0] = sm.u[rn];
+                w.u[1] = sm.u[rm];
+                w.u[2] = sm.u[r0];
+                w.s1 = s1;
+                w.beyond = wxy | (!P.per[2] ? (zo == 0 ? 16u : 0u) | (zo == P.nz - 1 ? 32u : 0u) : 0u);
+                scalars_compute_c<C, false>(P, D, x, y, zo, n, w, corr.a, corr.b);
+            } else {
+                // the stored value plus every increment of the step
+                // (correction, fluxes, sink) summed first: one rounding of the
+                // O(1) field
+                const R sink = Q.C != (R)0 ? kdc * om
+                                           : Q.kd * ((old.b + corr.b) - phi0_of(Q, old.a + corr.a));
+                ((F*)D.psi_dst)[n] = (F)(old.a + (corr.a + inc.a));
+                ((F*)D.phi_dst)[n] = (F)(old.b + ((corr.b + inc.b) - sink));
+            }
+        }
         r0 = r1;
     }
     cp_async_wait<0>();
 }
 
-// Resident blocks per SM of the transport: three (80 registers) measured
-// faster than four (64) on the 256^3 workload.
-constexpr int kScalBlocksPerSM = 3;
+// One block of kz_scalars, smem of scal_smem_bytes<C>() bytes.
+template <class C>
+__device__ __forceinline__ void kz_scalars_run(const DevParams& P, const DevPtrs& D, int x0, int y0, int z0, int nt,
+                                               unsigned char* smem_raw)
+{
+    using F = typename C::fld_t;
+    ScalSmem<F>& sm = *reinterpret_cast<ScalSmem<F>*>(smem_raw);
+    // the positions of this step's particle update stand in the records by now,
+    // and covering may be replacing the old ones: the old position lies within
+    // one step's velocity of the new one
+    find_solids<true>(P, D, x0, y0, 1, sm.sol, [](int, int, const DevPart&) {});
+    const bool xywall = beyond_xy(P, x0, y0, 1);
+    // planes any iteration looks at: z0 - 2 .. z0 + nt + 1
+    bool quiet = !xywall && (P.per[2] || (z0 >= 2 && z0 + nt + 2 <= P.nz));
+    for (int i = 0; i < sm.sol.n; ++i)
+        quiet = quiet && !spans_meet(sm.sol.lo[i], sm.sol.len[i], z0 - 2, nt + 4, P.nz, P.per[2]);
+    if (P.scheme) {
+        if (quiet)
+            scal_march<C, true, true>(P, D, x0, y0, z0, nt, xywall, sm);
+        else
+            scal_march<C, false, true>(P, D, x0, y0, z0, nt, xywall, sm);
+    } else {
+        if (quiet)
+            scal_march<C, true, false>(P, D, x0, y0, z0, nt, xywall, sm);
+        else
+            scal_march<C, false, false>(P, D, x0, y0, z0, nt, xywall, sm);
+    }
+}
 
 template <class C>
-__global__ void __launch_bounds__(kZThreads, kScalBlocksPerSM) kz_scalars(const __grid_constant__ DevParams P,
-                                                                          const __grid_constant__ DevPtrs D)
+constexpr size_t scal_smem_bytes()
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];   // sizeof(ScalSmem<F>)
+    return sizeof(ScalSmem<typename C::fld_t>);
+}
+
+// Resident blocks per SM of the transport: three in FP32 (80 registers), two
+// in FP64.
+template <class C>
+constexpr int scal_blocks_per_sm()
+{
+    return sizeof(typename C::real) == 8 ? 2 : 3;
+}
+
+template <class C>
+__global__ void __launch_bounds__(kZThreads, scal_blocks_per_sm<C>()) kz_scalars(const __grid_constant__ DevParams P,
+                                                                                const __grid_constant__ DevPtrs D)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];   // scal_smem_bytes<C>()
     const int zc = zm_chunk(P.nz, gridDim.z);
     const int z0 = blockIdx.z * zc;
     const int nt = min(z0 + zc, P.nz) - z0;
