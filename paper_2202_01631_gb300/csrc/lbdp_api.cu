@@ -238,10 +238,12 @@ void update_sides(lb_handle* h)
         h->dp.side1[a] = s1;
         h->dp.side2[a] = s2;
     }
-    // blocks per particle: about one box node per thread, at most kMaxPartBlocks
+    // blocks per particle, at most kMaxPartBlocks: part_slots nodes of the link
+    // box per thread, one of the cover box
     const long long t1 = (long long)h->dp.side1[0] * h->dp.side1[1] * h->dp.side1[2];
     const long long t2 = (long long)h->dp.side2[0] * h->dp.side2[1] * h->dp.side2[2];
-    const long long b1 = (t1 + 255) / 256, b2 = (t2 + 255) / 256;
+    const int per = part_slots(h->prm.precision == LB_FP64) * kPartThreads;
+    const long long b1 = (t1 + per - 1) / per, b2 = (t2 + kCoverThreads - 1) / kCoverThreads;
     h->dp.nb1 = (int)(b1 < kMaxPartBlocks ? (b1 > 0 ? b1 : 1) : kMaxPartBlocks);
     h->dp.nb2 = (int)(b2 < kMaxPartBlocks ? (b2 > 0 ? b2 : 1) : kMaxPartBlocks);
 }

@@ -215,7 +215,7 @@ void rebuild(lbb_batch* b)
             for (int k = 0; k < kNumBatchCfgs; ++k) zmax[k] = std::max(zmax[k], zm_blocks(h->dp, kZChunks[k]));
             lmax = std::max(lmax, h->dp.np * h->dp.nb1);
             cmax = std::max(cmax, h->dp.np * h->dp.nb2);
-            pmax = std::max(pmax, h->dp.np * pt_part_blocks(h->dp));
+            pmax = std::max(pmax, h->dp.np * pt_part_blocks(h->dp, b->precision == LB_FP64));
         }
         for (int k = 0; k < kNumBatchCfgs; ++k) pl.zgrid[k] = dim3(zmax[k], pl.L.nbox);
         pl.link = dim3(lmax, pl.L.nbox);

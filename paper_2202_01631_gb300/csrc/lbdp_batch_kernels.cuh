@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(kZThreads, scal_blocks_per_sm<C>()) kbz_scalar
 template <class C>
 __global__ void __launch_bounds__(kPartThreads, part_blocks_per_sm<C>()) kb_links(const __grid_constant__ BoxLaunch L)
 {
-    __shared__ LinkSmem<typename C::real> sm;
+    __shared__ LinkSmem<C> sm;
     const int b = blockIdx.y;
     if (b >= L.nbox || L.left[L.base + b] <= 0) return;
     const DevParams& P = L.box[b].P;
@@ -115,11 +115,11 @@ __global__ void __launch_bounds__(kPartThreads, part_blocks_per_sm<C>()) kb_link
 template <class C>
 __global__ void __launch_bounds__(kPartThreads) kb_pt_part(const __grid_constant__ BoxLaunch L)
 {
-    __shared__ NodeList list;
+    __shared__ NodeList<C> list;
     const int b = blockIdx.y;
     if (b >= L.nbox || L.left[L.base + b] <= 0) return;
     const DevParams& P = L.box[b].P;
-    const int nb = pt_part_blocks(P);
+    const int nb = pt_part_blocks(P, sizeof(typename C::real) == 8);
     const int p = blockIdx.x / nb, bi = blockIdx.x % nb;
     if (p >= P.np) return;
     pt_part_block<C>(P, L.box[b].D[L.par], p, bi, nb, list);
@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kPartThreads) kb_pt_part(const __grid_constant
 template <class C>
 __global__ void __launch_bounds__(kPartThreads) kb_f_part(const __grid_constant__ BoxLaunch L)
 {
-    __shared__ NodeList list;
+    __shared__ NodeList<C> list;
     const int b = blockIdx.y;
     if (b >= L.nbox || L.left[L.base + b] <= 0) return;
     const DevParams& P = L.box[b].P;
@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(kPartThreads) kb_f_part(const __grid_constant_
 template <class C>
 __global__ void __launch_bounds__(kPartThreads, part_blocks_per_sm<C>()) kb_collide_particles(const __grid_constant__ BoxLaunch L)
 {
-    __shared__ ColSmem<typename C::real> sm;
+    __shared__ ColSmem<C> sm;
     const int b = blockIdx.y;
     if (b >= L.nbox || L.left[L.base + b] <= 0) return;
     const DevParams& P = L.box[b].P;
@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(kPartThreads, part_blocks_per_sm<C>()) kb_coll
 template <class C>
 __global__ void __launch_bounds__(kPartThreads, part_blocks_per_sm<C>()) kb_scalars_particles(const __grid_constant__ BoxLaunch L)
 {
-    __shared__ NodeList list;
+    __shared__ NodeList<C> list;
     const int b = blockIdx.y;
     if (b >= L.nbox || L.left[L.base + b] <= 0) return;
     const DevParams& P = L.box[b].P;
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kPartThreads, part_blocks_per_sm<C>()) kb_scal
 }
 
 template <class C>
-__global__ void __launch_bounds__(kPartThreads) kb_cover_mark(const __grid_constant__ BoxLaunch L)
+__global__ void __launch_bounds__(kCoverThreads) kb_cover_mark(const __grid_constant__ BoxLaunch L)
 {
     const int b = blockIdx.y;
     if (b >= L.nbox || L.left[L.base + b] <= 0) return;
@@ -173,9 +173,9 @@ __global__ void __launch_bounds__(kPartThreads) kb_cover_mark(const __grid_const
 }
 
 template <class C>
-__global__ void __launch_bounds__(kPartThreads) kb_cover_apply(const __grid_constant__ BoxLaunch L)
+__global__ void __launch_bounds__(kCoverThreads) kb_cover_apply(const __grid_constant__ BoxLaunch L)
 {
-    __shared__ double smem[block_rows_bytes<kCoverK>(kPartThreads) / sizeof(double)];
+    __shared__ double smem[block_rows_bytes<kCoverK>(kCoverThreads) / sizeof(double)];
     __shared__ bool last;
     const int b = blockIdx.y;
     if (b >= L.nbox || L.left[L.base + b] <= 0) return;

@@ -49,7 +49,13 @@ using CfgF16 = Cfg<__half, float, float>;
 using CfgBF16 = Cfg<__nv_bfloat16, float, float>;
 
 constexpr int kRowThreads = 128;
-constexpr int kPartThreads = 256;
+// Threads of the kernels next to particles and of the covering kernels, and
+// the box slots a thread of the former looks at.  About a tenth of a sphere's
+// box lies next to it: a block of 128 threads finds the nodes of a full warp or
+// two and takes a quarter of the registers of an SM.  FP64 takes fewer blocks:
+// what they compute is taken from the bulk kernels on the same SM's FP64 pipe.
+constexpr int kPartThreads = 128, kCoverThreads = 256;
+__host__ __device__ constexpr int part_slots(bool fp64) { return fp64 ? 8 : 2; }
 
 constexpr uint8_t kWallSlot = 0xFF;    // slot beyond a non-periodic wall
 
@@ -675,11 +681,17 @@ __device__ __forceinline__ void rotate_unit(const double m[3], const double w[3]
     const double w2 = dot_x(w[0], w[1], w[2], w[0], w[1], w[2]);
     double s1, c1, cw;
     if (w2 < 0.01) {
-        s1 = fma_x(-w2 / 6.0, fma_x(-w2 / 20.0, fma_x(-w2 / 42.0, fma_x(-w2 / 72.0, fma_x(-w2 / 110.0, 1.0, 1.0),
-                                                                       1.0), 1.0), 1.0), 1.0);
-        c1 = 0.5 * fma_x(-w2 / 12.0, fma_x(-w2 / 30.0, fma_x(-w2 / 56.0, fma_x(-w2 / 90.0, fma_x(-w2 / 132.0, 1.0,
-                                                                                                  1.0), 1.0), 1.0),
-                                        1.0), 1.0);
+        // products with the rounded reciprocals: the divisions would be ten
+        // dependent chains on the FP64 pipe
+        s1 = fma_x(-w2 * (1.0 / 6.0),
+                   fma_x(-w2 * (1.0 / 20.0),
+                         fma_x(-w2 * (1.0 / 42.0),
+                               fma_x(-w2 * (1.0 / 72.0), fma_x(-w2 * (1.0 / 110.0), 1.0, 1.0), 1.0), 1.0), 1.0), 1.0);
+        c1 = 0.5 * fma_x(-w2 * (1.0 / 12.0),
+                         fma_x(-w2 * (1.0 / 30.0),
+                               fma_x(-w2 * (1.0 / 56.0),
+                                     fma_x(-w2 * (1.0 / 90.0), fma_x(-w2 * (1.0 / 132.0), 1.0, 1.0), 1.0), 1.0), 1.0),
+                         1.0);
         cw = fma_x(-w2, c1, 1.0);
     } else {
         const double wn = sqrt(w2);
@@ -1233,15 +1245,15 @@ __device__ __forceinline__ void cover_apply_block(const DevParams& P, const DevP
 // lbdp_zmarch.cuh)
 // ---------------------------------------------------------------------------
 template <class C>
-__global__ void __launch_bounds__(kPartThreads) k_cover_mark(DevParams P, DevPtrs D)
+__global__ void __launch_bounds__(kCoverThreads) k_cover_mark(DevParams P, DevPtrs D)
 {
     cover_mark_block<C>(P, D, blockIdx.y, blockIdx.x, gridDim.x);
 }
 
 template <class C>
-__global__ void __launch_bounds__(kPartThreads) k_cover_apply(DevParams P, DevPtrs D)
+__global__ void __launch_bounds__(kCoverThreads) k_cover_apply(DevParams P, DevPtrs D)
 {
-    __shared__ double smem[block_rows_bytes<kCoverK>(kPartThreads) / sizeof(double)];
+    __shared__ double smem[block_rows_bytes<kCoverK>(kCoverThreads) / sizeof(double)];
     __shared__ bool last;
     cover_apply_block<C>(P, D, blockIdx.y, blockIdx.x, gridDim.x, smem, last);
 }

@@ -31,13 +31,12 @@ inline cudaError_t set_carveout(const void* fn, int blocks, size_t smem)
 // attribute, so that it keeps the priority inside captured graphs too.
 // The same on another stream of the side group.
 template <class... A>
-inline void side_launch_on(cudaStream_t st, void (*k)(A...), dim3 grid, size_t smem, const SideStream* side,
+inline void side_launch_on(cudaStream_t st, void (*k)(A...), dim3 grid, int threads, const SideStream* side,
                            A... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
-    cfg.blockDim = dim3(kPartThreads);
-    cfg.dynamicSmemBytes = smem;
+    cfg.blockDim = dim3(threads);
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributePriority;
@@ -48,12 +47,11 @@ inline void side_launch_on(cudaStream_t st, void (*k)(A...), dim3 grid, size_t s
 }
 
 template <class... A>
-inline void side_launch(void (*k)(A...), dim3 grid, size_t smem, const SideStream* side, A... args)
+inline void side_launch(void (*k)(A...), dim3 grid, int threads, const SideStream* side, A... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
-    cfg.blockDim = dim3(kPartThreads);
-    cfg.dynamicSmemBytes = smem;
+    cfg.blockDim = dim3(threads);
     cfg.stream = side->s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributePriority;
@@ -87,7 +85,7 @@ struct Ops {
         return e;
     }
 
-    static dim3 pt_grid(const DevParams& P) { return dim3(pt_part_blocks(P), P.np); }
+    static dim3 pt_grid(const DevParams& P) { return dim3(pt_part_blocks(P, sizeof(R) == 8), P.np); }
 
     // One time step.  With particles and side streams: the particle kernels
     // (pressure tensor and force next to the particles, link sums and the
@@ -107,25 +105,25 @@ struct Ops {
         if (P.np > 0 && side && !ev) {
             cudaEventRecord(side->fork, s);
             cudaStreamWaitEvent(side->s2, side->fork, 0);
-            side_launch_on(side->s2, k_links<C>, pg1, 0, side, P, D);
+            side_launch_on(side->s2, k_links<C>, pg1, kPartThreads, side, P, D);
             cudaEventRecord(side->links_done, side->s2);
-            side_launch_on(side->s2, k_cover_mark<C>, pg2, 0, side, P, D);
+            side_launch_on(side->s2, k_cover_mark<C>, pg2, kCoverThreads, side, P, D);
             cudaEventRecord(side->mark_done, side->s2);
             cudaStreamWaitEvent(side->s, side->fork, 0);
-            side_launch(k_pt_part<C>, pgt, 0, side, P, D);
-            side_launch(k_f_part<C>, pg1, 0, side, P, D);
+            side_launch(k_pt_part<C>, pgt, kPartThreads, side, P, D);
+            side_launch(k_f_part<C>, pg1, kPartThreads, side, P, D);
             cudaStreamWaitEvent(side->s, side->links_done, 0);
-            side_launch(k_collide_particles<C>, pg1, 0, side, P, D);
+            side_launch(k_collide_particles<C>, pg1, kPartThreads, side, P, D);
             cudaEventRecord(side->bnd_done, side->s);
             kz_fused<C><<<g.zgrid, kZThreads, kFusedSmem, s>>>(P, D);
             cudaEventRecord(side->collide_done, s);
             cudaStreamWaitEvent(side->s, side->collide_done, 0);
-            side_launch(k_scalars_particles<C>, pg1, 0, side, P, D);
+            side_launch(k_scalars_particles<C>, pg1, kPartThreads, side, P, D);
             cudaStreamWaitEvent(side->s, side->mark_done, 0);
             // covering touches only nodes next to particles, whose fields the
             // side-stream kernels wrote, and leaves the next step's uniform
             // correction in the other buffer: it runs beside the transport
-            side_launch(k_cover_apply<C>, pg2, 0, side, P, D);
+            side_launch(k_cover_apply<C>, pg2, kCoverThreads, side, P, D);
             cudaEventRecord(side->scal_done, side->s);
             cudaStreamWaitEvent(s, side->bnd_done, 0);
             kz_scalars<C><<<g.zgrid_s, kZThreads, kZScalSmem, s>>>(P, D);
@@ -147,8 +145,8 @@ struct Ops {
         if (P.np > 0) k_scalars_particles<C><<<pg1, kPartThreads, 0, s>>>(P, D);
         if (ev) cudaEventRecord(ev[4], s);
         if (P.np > 0) {
-            k_cover_mark<C><<<pg2, kPartThreads, 0, s>>>(P, D);
-            k_cover_apply<C><<<pg2, kPartThreads, 0, s>>>(P, D);
+            k_cover_mark<C><<<pg2, kCoverThreads, 0, s>>>(P, D);
+            k_cover_apply<C><<<pg2, kCoverThreads, 0, s>>>(P, D);
         }
         if (ev) cudaEventRecord(ev[5], s);
         return cudaGetLastError();
@@ -295,22 +293,22 @@ struct BOps {
                 // s2 beside the force and boundary collide on s
                 cudaEventRecord(side->fork, s);
                 cudaStreamWaitEvent(side->s2, side->fork, 0);
-                side_launch_on(side->s2, kb_links<C>, L->link, 0, side, L->L);
+                side_launch_on(side->s2, kb_links<C>, L->link, kPartThreads, side, L->L);
                 cudaEventRecord(side->links_done, side->s2);
-                side_launch_on(side->s2, kb_cover_mark<C>, L->cover, 0, side, L->L);
+                side_launch_on(side->s2, kb_cover_mark<C>, L->cover, kCoverThreads, side, L->L);
                 cudaEventRecord(side->mark_done, side->s2);
                 cudaStreamWaitEvent(side->s, side->fork, 0);
-                side_launch(kb_pt_part<C>, L->ptg, 0, side, L->L);
-                side_launch(kb_f_part<C>, L->link, 0, side, L->L);
+                side_launch(kb_pt_part<C>, L->ptg, kPartThreads, side, L->L);
+                side_launch(kb_f_part<C>, L->link, kPartThreads, side, L->L);
                 cudaStreamWaitEvent(side->s, side->links_done, 0);
-                side_launch(kb_collide_particles<C>, L->link, 0, side, L->L);
+                side_launch(kb_collide_particles<C>, L->link, kPartThreads, side, L->L);
                 cudaEventRecord(side->bnd_done, side->s);
                 if ((e = node(0, cfg[0], L, s)) != cudaSuccess) return e;
                 cudaEventRecord(side->collide_done, s);
                 cudaStreamWaitEvent(side->s, side->collide_done, 0);
-                side_launch(kb_scalars_particles<C>, L->link, 0, side, L->L);
+                side_launch(kb_scalars_particles<C>, L->link, kPartThreads, side, L->L);
                 cudaStreamWaitEvent(side->s, side->mark_done, 0);
-                side_launch(kb_cover_apply<C>, L->cover, 0, side, L->L);
+                side_launch(kb_cover_apply<C>, L->cover, kCoverThreads, side, L->L);
                 cudaEventRecord(side->scal_done, side->s);
                 cudaStreamWaitEvent(s, side->bnd_done, 0);
                 if ((e = node(1, cfg[1], L, s)) != cudaSuccess) return e;
@@ -323,8 +321,8 @@ struct BOps {
                 if ((e = node(0, cfg[0], L, s)) != cudaSuccess) return e;
                 if ((e = node(1, cfg[1], L, s)) != cudaSuccess) return e;
                 kb_scalars_particles<C><<<L->link, kPartThreads, 0, s>>>(L->L);
-                kb_cover_mark<C><<<L->cover, kPartThreads, 0, s>>>(L->L);
-                kb_cover_apply<C><<<L->cover, kPartThreads, 0, s>>>(L->L);
+                kb_cover_mark<C><<<L->cover, kCoverThreads, 0, s>>>(L->L);
+                kb_cover_apply<C><<<L->cover, kCoverThreads, 0, s>>>(L->L);
             }
         }
         kb_advance<<<(nbox + 255) / 256, 256, 0, s>>>(left, nbox);

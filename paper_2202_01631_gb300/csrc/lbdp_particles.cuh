@@ -21,48 +21,70 @@
 
 namespace lbdp {
 
-// Blocks per SM the long bodies are compiled for: in FP32 arithmetic two, so
-// that a block fits beside one of kz_fused (128 registers); one in FP64.
+// Blocks per SM the long bodies are compiled for: four in FP32 arithmetic (128
+// registers), two in FP64, so that two or one fit in the place of a block of
+// kz_fused and need not wait for an SM of their own.
 template <class C>
 constexpr int part_blocks_per_sm()
 {
-    return sizeof(typename C::real) == 8 ? 1 : 2;
+    return sizeof(typename C::real) == 8 ? 2 : 4;
 }
 
 // ---------------------------------------------------------------------------
 // lists of nodes
 // ---------------------------------------------------------------------------
+constexpr int kScanWarps = kPartThreads / 32;
+template <class C>
 struct NodeList {
-    int n[kPartThreads];          // node indices, in box order
-    int wcount[kPartThreads / 32];
+    static constexpr int kScanSlots = part_slots(sizeof(typename C::real) == 8);
+    int n[kScanSlots * kPartThreads];   // node indices, in the order of the scan
+    int wcount[kScanSlots][kScanWarps];
 };
 
-// List the nodes of box slots t0 .. t0 + blockDim.x - 1 (edges s, origin o)
-// that pred(n, x, y, z) takes; returns their number.  Block-wide.
-template <class Pred>
-__device__ __forceinline__ int list_nodes(const DevParams& P, const int o[3], const int s[3], int t0, int tot,
-                                          NodeList& L, Pred pred)
+// List the nodes among the kScanSlots * blockDim.x box slots of block bi of
+// nbi, round r (edges s, origin o), that pred(n, x, y, z) takes; returns their
+// number.  Block-wide.  A block takes every nbi-th slot: consecutive ones would
+// give the blocks that hold a polar cap of the sphere many times the nodes of
+// the others.
+template <class C, class Pred>
+__device__ __forceinline__ int list_nodes(const DevParams& P, const int o[3], const int s[3], int r, int bi, int nbi,
+                                          int tot, NodeList<C>& L, Pred pred)
 {
+    constexpr int kScanSlots = NodeList<C>::kScanSlots;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int t = t0 + threadIdx.x;
-    int x, y, z, n = 0;
-    bool ok = t < tot && box_node(P, o, s, t, x, y, z);
-    if (ok) {
-        n = x + P.nx * (y + P.ny * z);
-        ok = pred(n, x, y, z);
-    }
-    const unsigned bal = __ballot_sync(0xffffffffu, ok);
-    __syncthreads();   // the list of the round before has been read
-    if (lane == 0) L.wcount[warp] = __popc(bal);
-    __syncthreads();
-    int base = 0, total = 0;
+    int n[kScanSlots];
+    bool ok[kScanSlots];
 #pragma unroll
-    for (int w = 0; w < kPartThreads / 32; ++w) {
-        const int c = L.wcount[w];
-        base += w < warp ? c : 0;
-        total += c;
+    for (int j = 0; j < kScanSlots; ++j) {
+        const int t = ((r * kScanSlots + j) * kPartThreads + (int)threadIdx.x) * nbi + bi;
+        int x, y, z;
+        n[j] = 0;
+        ok[j] = t < tot && box_node(P, o, s, t, x, y, z);
+        if (ok[j]) {
+            n[j] = x + P.nx * (y + P.ny * z);
+            ok[j] = pred(n[j], x, y, z);
+        }
     }
-    if (ok) L.n[base + __popc(bal & ((1u << lane) - 1u))] = n;
+    unsigned bal[kScanSlots];
+#pragma unroll
+    for (int j = 0; j < kScanSlots; ++j) bal[j] = __ballot_sync(0xffffffffu, ok[j]);
+    __syncthreads();   // the list of the round before has been read
+    if (lane == 0)
+#pragma unroll
+        for (int j = 0; j < kScanSlots; ++j) L.wcount[j][warp] = __popc(bal[j]);
+    __syncthreads();
+    int total = 0;
+#pragma unroll
+    for (int j = 0; j < kScanSlots; ++j) {
+        int base = total;
+#pragma unroll
+        for (int w = 0; w < kScanWarps; ++w) {
+            const int c = L.wcount[j][w];
+            base += w < warp ? c : 0;
+            total += c;
+        }
+        if (ok[j]) L.n[base + __popc(bal[j] & ((1u << lane) - 1u))] = n[j];
+    }
     __syncthreads();
     return total;
 }
@@ -221,8 +243,8 @@ __device__ __forceinline__ void pt_box(const DevParams& P, const DevPart& q, int
     }
 }
 
-// Blocks per particle of k_pt_part (about one node of the box per thread).
-__host__ __device__ inline int pt_part_blocks(const DevParams& P)
+// Blocks per particle of k_pt_part.
+__host__ __device__ inline int pt_part_blocks(const DevParams& P, bool fp64)
 {
     long long t = 1;
     const int L[3] = {P.nx, P.ny, P.nz};
@@ -231,7 +253,8 @@ __host__ __device__ inline int pt_part_blocks(const DevParams& P)
         if (P.per[a] && s > L[a]) s = L[a];
         t *= s;
     }
-    const long long b = (t + kPartThreads - 1) / kPartThreads;
+    const int per = part_slots(fp64) * kPartThreads;
+    const long long b = (t + per - 1) / per;
     return (int)(b < 1 ? 1 : (b > kMaxPartBlocks ? kMaxPartBlocks : b));
 }
 
@@ -241,7 +264,7 @@ __host__ __device__ inline int pt_part_blocks(const DevParams& P)
 // with the same values.
 template <class C>
 __device__ __forceinline__ void pt_part_block(const DevParams& P, const DevPtrs& D, int p, int bi, int nbi,
-                                              NodeList& list)
+                                              NodeList<C>& list)
 {
     using R = typename C::real;
     using F = typename C::fld_t;
@@ -253,28 +276,29 @@ __device__ __forceinline__ void pt_part_block(const DevParams& P, const DevPtrs&
     pt_box(P, q, o, sd);
     const int tot = sd[0] * sd[1] * sd[2];
     const size_t N = (size_t)P.N;
-    for (int t0 = bi * (int)blockDim.x; t0 < tot; t0 += nbi * (int)blockDim.x) {
-        const int cnt = list_nodes(P, o, sd, t0, tot, list, [&](int n, int x, int y, int z) {
+    for (int r = 0; (long long)r * NodeList<C>::kScanSlots * kPartThreads * nbi < tot; ++r) {
+        const int cnt = list_nodes(P, o, sd, r, bi, nbi, tot, list, [&](int n, int x, int y, int z) {
             int Dn[3];
             int_offset(P, g, x, y, z, Dn);
             const float d0 = (float)Dn[0] - g.fr[0], d1 = (float)Dn[1] - g.fr[1], d2 = (float)Dn[2] - g.fr[2];
             return dot_x(d0, d1, d2, d0, d1, d2) < reach * reach && D.mask[n] == 0;
         });
-        if ((int)threadIdx.x >= cnt) continue;
-        const int n = list.n[threadIdx.x];
-        int x, y, z;
-        node_coords(P, n, x, y, z);
-        GAcc<F, 2> a;
-        neighbours(P, x, y, z, a.nb);
-        a.n = n;
-        a.mk = D.mask;
-        a.f[0] = (const F*)D.psi_src;
-        a.f[1] = (const F*)D.phi_src;
-        R mps, mph, pt[kPtFields];
-        mup_values<C>(P, D, x, y, z, a, corr_r<R>(D, 0), corr_r<R>(D, 1), mps, mph, pt);
-        F* ptg = (F*)D.pt;
+        for (int e = threadIdx.x; e < cnt; e += kPartThreads) {
+            const int n = list.n[e];
+            int x, y, z;
+            node_coords(P, n, x, y, z);
+            GAcc<F, 2> a;
+            neighbours(P, x, y, z, a.nb);
+            a.n = n;
+            a.mk = D.mask;
+            a.f[0] = (const F*)D.psi_src;
+            a.f[1] = (const F*)D.phi_src;
+            R mps, mph, pt[kPtFields];
+            mup_values<C>(P, D, x, y, z, a, corr_r<R>(D, 0), corr_r<R>(D, 1), mps, mph, pt);
+            F* ptg = (F*)D.pt;
 #pragma unroll
-        for (int k = 0; k < kPtFields; ++k) ptg[k * N + n] = (F)pt[k];
+            for (int k = 0; k < kPtFields; ++k) ptg[k * N + n] = (F)pt[k];
+        }
     }
 }
 
@@ -282,7 +306,7 @@ template <class C>
 __global__ void __launch_bounds__(kPartThreads) k_pt_part(const __grid_constant__ DevParams P,
                                                            const __grid_constant__ DevPtrs D)
 {
-    __shared__ NodeList list;
+    __shared__ NodeList<C> list;
     pt_part_block<C>(P, D, blockIdx.y, blockIdx.x, gridDim.x, list);
 }
 
@@ -298,30 +322,31 @@ __device__ __forceinline__ void link_box(const DevPart& q, int o[3])
 // particle is p, as in k_collide_particles), into the force array.
 template <class C>
 __device__ __forceinline__ void f_part_block(const DevParams& P, const DevPtrs& D, int p, int bi, int nbi,
-                                             NodeList& list)
+                                             NodeList<C>& list)
 {
     using F = typename C::fld_t;
     int o[3];
     link_box(D.parts[p], o);
     const int tot = P.side1[0] * P.side1[1] * P.side1[2];
-    for (int t0 = bi * (int)blockDim.x; t0 < tot; t0 += nbi * (int)blockDim.x) {
-        const int cnt = list_nodes(P, o, P.side1, t0, tot, list,
+    for (int r = 0; (long long)r * NodeList<C>::kScanSlots * kPartThreads * nbi < tot; ++r) {
+        const int cnt = list_nodes(P, o, P.side1, r, bi, nbi, tot, list,
                                    [&](int n, int, int, int) { return D.mask[n] == 0 && D.bflag[n] != 0; });
-        if ((int)threadIdx.x >= cnt) continue;
-        const int n = list.n[threadIdx.x];
-        int x, y, z;
-        node_coords(P, n, x, y, z);
-        // a node next to several particles: each of their blocks writes the
-        // same force
-        const size_t N = (size_t)P.N;
-        const F* pt = (const F*)D.pt;
-        GAcc<F, kPtFields> a;
-        neighbours(P, x, y, z, a.nb);
-        a.n = n;
-        a.mk = D.mask;
+        for (int e = threadIdx.x; e < cnt; e += kPartThreads) {
+            const int n = list.n[e];
+            int x, y, z;
+            node_coords(P, n, x, y, z);
+            // a node next to several particles: each of their blocks writes the
+            // same force
+            const size_t N = (size_t)P.N;
+            const F* pt = (const F*)D.pt;
+            GAcc<F, kPtFields> a;
+            neighbours(P, x, y, z, a.nb);
+            a.n = n;
+            a.mk = D.mask;
 #pragma unroll
-        for (int k = 0; k < kPtFields; ++k) a.f[k] = pt + k * N;
-        fdiv_compute<C>(P, D, n, a);
+            for (int k = 0; k < kPtFields; ++k) a.f[k] = pt + k * N;
+            fdiv_compute<C>(P, D, n, a);
+        }
     }
 }
 
@@ -329,7 +354,7 @@ template <class C>
 __global__ void __launch_bounds__(kPartThreads) k_f_part(const __grid_constant__ DevParams P,
                                                           const __grid_constant__ DevPtrs D)
 {
-    __shared__ NodeList list;
+    __shared__ NodeList<C> list;
     f_part_block<C>(P, D, blockIdx.y, blockIdx.x, gridDim.x, list);
 }
 
@@ -363,12 +388,13 @@ __global__ void __launch_bounds__(kPartThreads) k_f_part(const __grid_constant__
 // Measured on GB300, FP32, one sphere R = 8: 56 us with 41 FP64 sums over the
 // links (250 registers, 84 KB of shared memory).
 // ---------------------------------------------------------------------------
-constexpr int kRowF = 20, kRowI = 27, kRow = kRowF + kRowI, kRowGroups = 5, kRowNodes = 64;
+constexpr int kRowF = 20, kRowI = 27, kRow = kRowF + kRowI, kRowGroups = 2, kRowNodes = 64;
 static_assert(kRowGroups * kRow <= kPartThreads, "a thread per column and group of rows");
 
-template <class R>
+template <class C>
 struct LinkSmem {
-    NodeList list;
+    using R = typename C::real;
+    NodeList<C> list;
     DevPart part;
     R rf[kRowNodes][kRowF + 1];
     int ri[kRowNodes][kRowI];
@@ -565,7 +591,7 @@ __device__ __forceinline__ double zeta_entry(int a, int b, const double* Z, cons
 // batched kernels, so both give identical bits.
 template <class C>
 __device__ __forceinline__ void links_block(const DevParams& P, const DevPtrs& D, int p, int bi, int nbi,
-                                            LinkSmem<typename C::real>& sm)
+                                            LinkSmem<C>& sm)
 {
     constexpr int K = kLinkK;
     {   // the particle's record, by the whole block
@@ -582,8 +608,8 @@ __device__ __forceinline__ void links_block(const DevParams& P, const DevPtrs& D
     const int col = threadIdx.x % kRow, grp = threadIdx.x / kRow;
     double accf = 0.0;
     long long acci = 0;
-    for (int t0 = bi * (int)blockDim.x; t0 < tot; t0 += nbi * (int)blockDim.x) {
-        const int cnt = list_nodes(P, o, P.side1, t0, tot, sm.list,
+    for (int r = 0; (long long)r * NodeList<C>::kScanSlots * kPartThreads * nbi < tot; ++r) {
+        const int cnt = list_nodes(P, o, P.side1, r, bi, nbi, tot, sm.list,
                                    [&](int n, int, int, int) { return D.mask[n] == 0 && D.bflag[n] != 0; });
         for (int s0 = 0; s0 < cnt; s0 += kRowNodes) {
             const int m = min(cnt - s0, kRowNodes);
@@ -671,7 +697,7 @@ template <class C>
 __global__ void __launch_bounds__(kPartThreads, part_blocks_per_sm<C>()) k_links(const __grid_constant__ DevParams P,
                                                          const __grid_constant__ DevPtrs D)
 {
-    __shared__ LinkSmem<typename C::real> sm;
+    __shared__ LinkSmem<C> sm;
     links_block<C>(P, D, blockIdx.y, blockIdx.x, gridDim.x, sm);
 }
 
@@ -680,17 +706,18 @@ __global__ void __launch_bounds__(kPartThreads, part_blocks_per_sm<C>()) k_links
 // with u_b = U + Omega x r + v_s on particle links.  A node next to several
 // particles is collided by the lowest of them.
 // ---------------------------------------------------------------------------
-constexpr int kColNodes = 128;   // nodes of a round: one per thread of half a block
+constexpr int kColNodes = kPartThreads;   // nodes of a round
 
-template <class R>
+template <class C>
 struct ColSmem {
-    NodeList list;
+    using R = typename C::real;
+    NodeList<C> list;
     R cub[19][kColNodes];   // 6 w rho0 c . u_b of the links of each node
 };
 
 template <class C>
 __device__ __forceinline__ void collide_particles_block(const DevParams& P, const DevPtrs& D, int p, int bi, int nbi,
-                                                        ColSmem<typename C::real>& sm)
+                                                        ColSmem<C>& sm)
 {
     using R = typename C::real;
     using F = typename C::fld_t;
@@ -704,12 +731,12 @@ __device__ __forceinline__ void collide_particles_block(const DevParams& P, cons
     int o[3];
     link_box(D.parts[p], o);
     const int tot = P.side1[0] * P.side1[1] * P.side1[2];
-    for (int t0 = bi * (int)blockDim.x; t0 < tot; t0 += nbi * (int)blockDim.x) {
-        const int cnt = list_nodes(P, o, P.side1, t0, tot, sm.list,
+    for (int r = 0; (long long)r * NodeList<C>::kScanSlots * kPartThreads * nbi < tot; ++r) {
+        const int cnt = list_nodes(P, o, P.side1, r, bi, nbi, tot, sm.list,
                                    [&](int n, int, int, int) { return D.mask[n] == 0 && D.bflag[n] != 0; });
         for (int s0 = 0; s0 < cnt; s0 += kColNodes) {
             const int t = (int)threadIdx.x;
-            if (t >= kColNodes || s0 + t >= cnt) continue;
+            if (s0 + t >= cnt) continue;
             const int n = sm.list.n[s0 + t];
             int x, y, z;
             node_coords(P, n, x, y, z);
@@ -766,7 +793,7 @@ template <class C>
 __global__ void __launch_bounds__(kPartThreads, part_blocks_per_sm<C>()) k_collide_particles(const __grid_constant__ DevParams P,
                                                                      const __grid_constant__ DevPtrs D)
 {
-    __shared__ ColSmem<typename C::real> sm;
+    __shared__ ColSmem<C> sm;
     collide_particles_block<C>(P, D, blockIdx.y, blockIdx.x, gridDim.x, sm);
 }
 
@@ -791,58 +818,59 @@ struct SAcc {
 
 template <class C>
 __device__ __forceinline__ void scalars_particles_block(const DevParams& P, const DevPtrs& D, int p, int bi, int nbi,
-                                                        NodeList& list)
+                                                        NodeList<C>& list)
 {
     using R = typename C::real;
     using F = typename C::fld_t;
     int o[3];
     link_box(D.parts[p], o);
     const int tot = P.side1[0] * P.side1[1] * P.side1[2];
-    for (int t0 = bi * (int)blockDim.x; t0 < tot; t0 += nbi * (int)blockDim.x) {
-        const int cnt = list_nodes(P, o, P.side1, t0, tot, list,
+    for (int r = 0; (long long)r * NodeList<C>::kScanSlots * kPartThreads * nbi < tot; ++r) {
+        const int cnt = list_nodes(P, o, P.side1, r, bi, nbi, tot, list,
                                    [&](int n, int, int, int) { return D.mask[n] == 0 && D.bflag[n] != 0; });
-        if ((int)threadIdx.x >= cnt) continue;
-        const int n = list.n[threadIdx.x];
-        int x, y, z;
-        node_coords(P, n, x, y, z);
-        Around a;
-        look_around(P, D, x, y, z, a);
-        if (a.lo != p + 1) continue;
-        SAcc<F> g;
+        for (int e = threadIdx.x; e < cnt; e += kPartThreads) {
+            const int n = list.n[e];
+            int x, y, z;
+            node_coords(P, n, x, y, z);
+            Around a;
+            look_around(P, D, x, y, z, a);
+            if (a.lo != p + 1) continue;
+            SAcc<F> g;
 #pragma unroll
-        for (int i = 0; i < 19; ++i) g.nb[i] = a.nb[i];
-        g.n = n;
-        g.mk = D.mask;
-        g.psi = (const F*)D.psi_src;
-        g.phi = (const F*)D.phi_src;
-        g.mu = (const F*)D.mu;
-        g.u = (const F*)D.u;
-        g.N = (int)P.N;
-        const R dps = corr_r<R>(D, 0), dph = corr_r<R>(D, 1);
-        const R ps = (R)g.psi[n] + dps, ph = (R)g.phi[n] + dph;
-        // links into particles: no diffusive flux; the scalars leave with the
-        // boundary velocity of the bounce-back rule, c.u_b g(x) -- weighted
-        // w_i on the D3Q19 links of the finite-difference scheme, 1 on the six
-        // D3Q7 links of the lattice-Boltzmann one; Janus production on the
-        // m.(x - X) <= 0 side of each adjacent particle (any of the 18)
-        R gphi[3];
-        grad_phi_around<R, F>(a, g.phi, n, ph, dph, gphi);
-        R out = 0, src = 0;   // sum of w c.u_b
-        for (int k = a.lo; k <= a.hi; ++k) {
-            unsigned b = links_into(a, k);
-            if (!b) continue;
-            const DevPart& q = D.parts[k - 1];
-            NodeLinks<R> l;
-            node_links<R>(P, q, x, y, z, l);
-            if (cap_minus_at(l.q, l.D, 0, 0, 0)) src += PartR<R>::alpha(q);
-            if (P.scheme) b &= 0x7Eu;
-            for (; b; b &= b - 1) {
-                const int i = __ffs((int)b) - 1;
-                const R w = P.scheme ? (R)1 : (i < 7 ? (R)(1.0 / 18.0) : (R)(1.0 / 36.0));
-                out = fma_x(w, link_cub<R>(l, i, gphi), out);
+            for (int i = 0; i < 19; ++i) g.nb[i] = a.nb[i];
+            g.n = n;
+            g.mk = D.mask;
+            g.psi = (const F*)D.psi_src;
+            g.phi = (const F*)D.phi_src;
+            g.mu = (const F*)D.mu;
+            g.u = (const F*)D.u;
+            g.N = (int)P.N;
+            const R dps = corr_r<R>(D, 0), dph = corr_r<R>(D, 1);
+            const R ps = (R)g.psi[n] + dps, ph = (R)g.phi[n] + dph;
+            // links into particles: no diffusive flux; the scalars leave with the
+            // boundary velocity of the bounce-back rule, c.u_b g(x) -- weighted
+            // w_i on the D3Q19 links of the finite-difference scheme, 1 on the six
+            // D3Q7 links of the lattice-Boltzmann one; Janus production on the
+            // m.(x - X) <= 0 side of each adjacent particle (any of the 18)
+            R gphi[3];
+            grad_phi_around<R, F>(a, g.phi, n, ph, dph, gphi);
+            R out = 0, src = 0;   // sum of w c.u_b
+            for (int k = a.lo; k <= a.hi; ++k) {
+                unsigned b = links_into(a, k);
+                if (!b) continue;
+                const DevPart& q = D.parts[k - 1];
+                NodeLinks<R> l;
+                node_links<R>(P, q, x, y, z, l);
+                if (cap_minus_at(l.q, l.D, 0, 0, 0)) src += PartR<R>::alpha(q);
+                if (P.scheme) b &= 0x7Eu;
+                for (; b; b &= b - 1) {
+                    const int i = __ffs((int)b) - 1;
+                    const R w = P.scheme ? (R)1 : (i < 7 ? (R)(1.0 / 18.0) : (R)(1.0 / 36.0));
+                    out = fma_x(w, link_cub<R>(l, i, gphi), out);
+                }
             }
+            scalars_compute_c<C, true>(P, D, x, y, z, n, g, dps, dph, mul_x(-out, ps), mul_x(-out, ph), src);
         }
-        scalars_compute_c<C, true>(P, D, x, y, z, n, g, dps, dph, mul_x(-out, ps), mul_x(-out, ph), src);
     }
 }
 
@@ -850,7 +878,7 @@ template <class C>
 __global__ void __launch_bounds__(kPartThreads, part_blocks_per_sm<C>()) k_scalars_particles(const __grid_constant__ DevParams P,
                                                                      const __grid_constant__ DevPtrs D)
 {
-    __shared__ NodeList list;
+    __shared__ NodeList<C> list;
     scalars_particles_block<C>(P, D, blockIdx.y, blockIdx.x, gridDim.x, list);
 }
 
