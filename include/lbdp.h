@@ -159,9 +159,10 @@ int lb_add_particle(lb_handle* h, const lb_particle_desc* desc, int* id_out);
  * force, streaming with bounce-back and BGK collision; psi/phi transport
  * (Eq. diffusion_reaction); particle update; covering/uncovering.  The
  * particle kernels run on a second stream of the library's that joins the
- * handle's stream before each step ends.  A box without particles runs whole
- * groups of 8 steps as one captured CUDA graph (captured on first use and
- * again after its parameters or launch grids change); while the caller is
+ * handle's stream before each step ends.  Whole groups of 8 steps run as one
+ * captured CUDA graph for a box without particles, and for a small one with
+ * particles once it has run 128 steps (captured on first use and again after
+ * the parameters or launch grids change); while the caller is
  * itself capturing the handle's stream, and on the legacy default stream,
  * every step is launched plainly.  Results do not depend on the route. */
 int lb_step(lb_handle* h, int nsteps);
@@ -195,9 +196,9 @@ int lb_profile_step(lb_handle* h, int nsteps, double* ms, int* launches);
  * times per launch (0 fused, 1 transport).  Synchronises.  LB_ERR_PARAM for
  * reps < 1. */
 int lb_tune(lb_handle* h, int reps, int planes_out[2], double ms_out[2]);
-/* Set the chunk lengths directly; 0 restores the size heuristic (a chunk
- * count of about six waves of four blocks per SM, chunks of at least 6
- * planes); lengths above nz are clamped.  LB_ERR_PARAM for a negative one. */
+/* Set the chunk lengths directly; 0 restores the library's choice by size (a
+ * cost model fitted to measured chunks); lengths above nz are clamped.
+ * LB_ERR_PARAM for a negative one. */
 int lb_set_planes(lb_handle* h, const int planes[2]);
 /* The chunk lengths the next lb_step uses (after rounding to equal chunks). */
 int lb_get_planes(const lb_handle* h, int planes[2]);

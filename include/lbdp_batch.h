@@ -84,7 +84,9 @@ int lbb_get_steps(const lbb_batch* b, const lb_handle* h, long long* left);
 
 /* Run nsteps batch steps: in each, every box with steps left advances one
  * time step.  Full chunks of graph_steps run as one captured CUDA graph (one
- * graph launch), the rest as plain launches.  Queued on the batch stream;
+ * graph launch) once the boxes have run four of them since the batch last
+ * changed, or when nsteps holds four; the rest as plain launches.  Queued on
+ * the batch stream;
  * returns without waiting.  launches (optional) receives the number of kernel
  * launches the call queued (graph nodes included). */
 int lbb_run(lbb_batch* b, int nsteps, long long* launches);

@@ -306,8 +306,20 @@ int read_err(lb_handle* h)
 }
 
 
-// Steps per captured graph of lb_step (even: a launch leaves the parity).
-constexpr int kGraphSteps = 8;
+// Steps per captured graph of lb_step (even: a launch leaves the parity), and
+// the steps a box with particles runs plainly before its graph is captured: the
+// capture of eight steps of nine kernels costs about as much as a hundred steps
+// gain by it.
+constexpr int kGraphSteps = 8, kGraphAfter = 128;
+
+// Whether graph launches beat plain ones.  Without particles they do (measured
+// on GB300: 170 instead of 174 us per step at 128^3).  With particles a step
+// has nine kernels on three streams; in a graph the edges between them cost
+// less, but the particle kernels lose some of their head start before the bulk
+// kernels.  Plain -> graph, us per step: FP32 24^3 70 -> 57, 40 x 38 x 44 71 ->
+// 61, 64^3 90 -> 84, 96^3 135 -> 118, 110 x 100 x 96 153 -> 156, 160 x 150 x 170
+// 283 -> 292; FP64 32^3 178 -> 172, 48^3 458 -> 482, 64^3 621 -> 617.
+bool graph_pays(const DevParams& P, bool fp64) { return P.np == 0 || P.N <= (fp64 ? 1ll << 15 : 1ll << 20); }
 
 bool same_grid(const dim3& a, const dim3& b) { return a.x == b.x && a.y == b.y && a.z == b.z; }
 
@@ -518,21 +530,20 @@ int lb_step(lb_handle* h, int nsteps)
     cudaSetDevice(h->device);
     const RowGrid g = row_grid(h);
     int t = 0;
-    // A box without particles runs whole groups of kGraphSteps steps as one
-    // graph launch each (measured on GB300: 170 instead of 174 us per step at
-    // 128^3); the graphs are captured again when the parameters or the launch
-    // grids have changed since.  With particles the step forks onto the side
-    // stream, and the captured form measured slower than the plain launches
-    // (283 instead of 245 us at 128^3 with one sphere, the side kernels'
-    // priority attribute notwithstanding), so those steps stay plain.
-    if (h->dp.np == 0 && nsteps >= kGraphSteps && can_capture(h)) {
+    // Groups of kGraphSteps steps as one graph launch each, where that pays; the
+    // graphs are captured again when the parameters or the launch grids have
+    // changed since.
+    if (nsteps >= kGraphSteps && graph_pays(h->dp, h->prm.precision == LB_FP64) && can_capture(h)) {
         if (memcmp(&h->g_dp, &h->dp, sizeof(DevParams)) != 0 || !same_grid(h->g_grid.zgrid, g.zgrid) ||
             !same_grid(h->g_grid.zgrid_s, g.zgrid_s)) {
             drop_step_graphs(h);
             memcpy(&h->g_dp, &h->dp, sizeof(DevParams));
             h->g_grid = g;
+            h->g_steps = 0;
         }
-        for (; nsteps - t >= kGraphSteps; t += kGraphSteps) {
+        const bool wait = h->dp.np > 0 && h->g_steps < kGraphAfter && nsteps < kGraphAfter;
+        h->g_steps += nsteps;
+        for (; !wait && nsteps - t >= kGraphSteps; t += kGraphSteps) {
             if (!h->gexec[h->cur]) {
                 const int st = capture_steps(h, g, h->cur);
                 if (st != LB_OK) return st;

@@ -163,6 +163,7 @@ struct lbb_batch {
     long long* d_left = nullptr;
     std::vector<LaunchPlan> plans;
     int par = 0;            // parity of the steps run since the plans were built
+    long long ran = 0;      // and their number
     int cfg[kNumBatchClasses] = {1, 1};   // z chunks of 16 planes until tuned
     cudaGraphExec_t exec[2] = {nullptr, nullptr};   // graphs starting at parity 0 / 1
     SideStream side{};   // particle kernels, overlapping the fluid kernels
@@ -223,6 +224,7 @@ void rebuild(lbb_batch* b)
         pl.ptg = dim3(pmax, pl.L.nbox);
     }
     b->par = 0;
+    b->ran = 0;
     b->dirty = false;
     drop_graph(b);
 }
@@ -464,7 +466,11 @@ int lbb_run(lbb_batch* b, int nsteps, long long* launches)
     if (plans_stale(b)) rebuild(b);
     int st = upload_counts(b, false);
     if (st != LB_OK) return st;
-    const int full = n / b->graph_steps, rest = n % b->graph_steps;
+    // a capture costs about as much as four runs of the graph gain by it: short
+    // runs between changes of the batch (requests that come and go) stay plain
+    const bool graph = n >= b->graph_steps && (b->exec[b->par] || n >= 4 * b->graph_steps ||
+                                               b->ran >= 4 * b->graph_steps);
+    const int full = graph ? n / b->graph_steps : 0, rest = n - full * b->graph_steps;
     if (full > 0) {
         st = capture_graph(b, b->par);
         if (st != LB_OK) return st;
@@ -473,6 +479,7 @@ int lbb_run(lbb_batch* b, int nsteps, long long* launches)
     for (int k = 0; k < rest && st == LB_OK; ++k) st = step(b, (b->par + k) & 1);
     if (st != LB_OK) return st;
     b->par = (b->par + n) & 1;
+    b->ran += n;
     for (Member& m : b->mem) {
         const long long ran = std::min<long long>(m.left, n);
         m.left -= ran;
