@@ -1066,11 +1066,24 @@ __device__ __forceinline__ void cover_mark_block(const DevParams& P, const DevPt
     }
 }
 
+// A kernel launched with programmatic stream serialization starts once every
+// block of the kernel before it in the stream has called release_next_grid (or
+// has ended), and may run its first part beside it; wait_for_prior_grid
+// returns when that kernel has ended and its writes are visible.  Both do
+// nothing in a kernel launched without the attribute.
+__device__ __forceinline__ void release_next_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 //
 // cover_apply_block runs block bi of the nbi blocks of particle p; the last of
 // the np * nbi blocks of the box (a ticket) finishes the step for all
 // particles of the box.  smem holds block_rows_bytes<kCoverK>(blockDim.x)
 // bytes.
+// Bound by latency: few nodes, a chain of dependent loads.  In most steps no node
+// of a block changes, and then it adds nothing up; the last block gives each
+// particle a warp instead of taking one after the other with all its threads
+// (alone: 11.1 -> 9.5 us with one sphere at 24^3, 29.1 -> 14.7 us with eight at
+// 256^3).
 template <class C>
 __device__ __forceinline__ void cover_apply_block(const DevParams& P, const DevPtrs& D, int p, int bi, int nbi,
                                                   double* smem, bool& last)
@@ -1092,6 +1105,7 @@ __device__ __forceinline__ void cover_apply_block(const DevParams& P, const DevP
     double acc[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) acc[k] = 0.0;
+    bool changed = false;
     for (int t = bi * blockDim.x + threadIdx.x; t < tot; t += nbi * blockDim.x) {
         int x, y, z;
         if (!box_node(P, o, P.side2, t, x, y, z)) continue;
@@ -1107,8 +1121,10 @@ __device__ __forceinline__ void cover_apply_block(const DevParams& P, const DevP
             const int m = nb[i] >= 0 ? nb[i] : n;
             adj = adj || (nb[i] >= 0 && D.mask_next[m]);
         }
+        wait_for_prior_grid();   // k_scalars_particles reads the old flags and writes the fields
         D.bflag[n] = (!nw && adj) ? 1 : 0;
         if (ob == nw) continue;
+        changed = true;
         if (ob == 0 && nw == p + 1) {
             // covered: the particle takes the momentum the node's populations
             // carry; psi, phi are removed
@@ -1190,46 +1206,74 @@ __device__ __forceinline__ void cover_apply_block(const DevParams& P, const DevP
             atomicOr(D.err, kErrOverlap);   // passed straight into another sphere
         }
     }
-    block_sum_rows<K>(acc, smem);
+    wait_for_prior_grid();   // threads without a node
     double* part = D.cover_part + ((size_t)p * kMaxPartBlocks + bi) * K;
+    const int any = __syncthreads_or(changed);
+    if (any) block_sum_rows<K>(acc, smem);
+    if ((int)threadIdx.x < K) part[threadIdx.x] = any ? smem[threadIdx.x] : 0.0;
+    __syncthreads();
     if (threadIdx.x == 0) {
-        for (int k = 0; k < K; ++k) part[k] = acc[k];
         __threadfence();
         last = (atomicAdd(D.cover_ticket, 1u) == (unsigned)(nbi * P.np) - 1u);
     }
     __syncthreads();
     if (!last) return;
-    // last block of the grid: per particle, thread b loads block b's partials
-    // and the block reduction adds them in a fixed order; impulses go to their
-    // particles, deficits into the uniform correction, particles move
+    // last block of the grid, one warp per particle: lane l adds the partials
+    // of blocks l, l + 32, ..., the lanes' sums meet in a fixed tree; impulses
+    // go to their particles, deficits into the uniform correction, particles
+    // move
     __threadfence();
-    double dsum_psi = 0.0, dsum_phi = 0.0, dcnt = 0.0;
-    for (int k = 0; k < P.np; ++k) {
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int k = threadIdx.x >> 5; k < P.np; k += nw) {
+        DevPart& dk = D.parts[k];
         double s[K];
 #pragma unroll
         for (int c = 0; c < K; ++c) s[c] = 0.0;
-        if ((int)threadIdx.x < nbi) {
-            const double* cp = D.cover_part + ((size_t)k * kMaxPartBlocks + threadIdx.x) * K;
+        for (int b = lane; b < nbi; b += 32) {
+            const double* cp = D.cover_part + ((size_t)k * kMaxPartBlocks + b) * K;
 #pragma unroll
-            for (int c = 0; c < K; ++c) s[c] = __ldcg(cp + c);
+            for (int c = 0; c < K; ++c) s[c] += __ldcg(cp + c);
         }
-        block_sum_rows<K>(s, smem);
-        if (threadIdx.x == 0) {
-            DevPart& dk = D.parts[k];
+        bool nz = false;
+#pragma unroll
+        for (int c = 0; c < K; ++c) nz = nz || s[c] != 0.0;
+        if (__any_sync(0xffffffffu, nz)) {
+            for (int w = 16; w > 0; w >>= 1)
+#pragma unroll
+                for (int c = 0; c < K; ++c) s[c] += __shfl_xor_sync(0xffffffffu, s[c], w);
+        }
+        if (lane == 0) {
+            // all loads first: a store after each load would wait for it
+            const Geo gn = dk.gn;
+            double X[3], m[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                X[a] = dk.Xn[a];
+                m[a] = dk.mn[a];
+            }
+            const double wp = dk.wall_psi, wh = dk.wall_phi;
+#pragma unroll
             for (int a = 0; a < 3; ++a) {
                 dk.imp_f[a] = s[a];
                 dk.imp_t[a] = s[3 + a];
-                dk.X[a] = dk.Xn[a];
-                dk.m[a] = dk.mn[a];
-                dk.mf[a] = (float)dk.mn[a];
+                dk.X[a] = X[a];
+                dk.m[a] = m[a];
+                dk.mf[a] = (float)m[a];
             }
-            dk.g = dk.gn;
-            dsum_psi += s[6] + dk.wall_psi;
-            dsum_phi += s[7] + dk.wall_phi;
-            dcnt += s[8];
+            dk.g = gn;
+            smem[3 * k] = s[6] + wp;
+            smem[3 * k + 1] = s[7] + wh;
+            smem[3 * k + 2] = s[8];
         }
     }
+    __syncthreads();
     if (threadIdx.x != 0) return;
+    double dsum_psi = 0.0, dsum_phi = 0.0, dcnt = 0.0;
+    for (int k = 0; k < P.np; ++k) {
+        dsum_psi += smem[3 * k];
+        dsum_phi += smem[3 * k + 1];
+        dcnt += smem[3 * k + 2];
+    }
     const long long nf = *D.nfluid + (long long)dcnt;
     *D.nfluid = nf;
     D.corr_next[0] = dsum_psi / (double)nf;

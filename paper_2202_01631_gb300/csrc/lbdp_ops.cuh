@@ -10,56 +10,51 @@
 
 namespace lbdp {
 
-// Shared-memory carve-out hint (percent of the SM's maximum) that leaves room
-// for `blocks` resident blocks of `smem` bytes each and gives the rest of the
-// SM's on-chip memory to L1, which serves the halo reloads of the tiled
-// stencils.  Without it the driver takes the largest carve-out the block count
-// allows and leaves L1 a few tens of KB.
-inline cudaError_t set_carveout(const void* fn, int blocks, size_t smem)
-{
-    int dev = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    if (e != cudaSuccess || per_sm <= 0) return e;
-    const size_t need = (size_t)blocks * (smem + 1024);   // 1 KB per block is reserved
-    long long pct = (long long)((100 * need + per_sm - 1) / per_sm);
-    if (pct > 100) pct = 100;
-    return cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, (int)pct);
-}
-
-// Launch of a side-stream kernel with the side stream's priority as a launch
+// Launch of a side-stream kernel with the side streams' priority as a launch
 // attribute, so that it keeps the priority inside captured graphs too.
-// The same on another stream of the side group.
 template <class... A>
-inline void side_launch_on(cudaStream_t st, void (*k)(A...), dim3 grid, int threads, const SideStream* side,
-                           A... args)
+inline void side_launch_with(cudaLaunchAttribute* at, int nat, cudaStream_t st, void (*k)(A...), dim3 grid,
+                             int threads, const SideStream* side, A... args)
 {
+    at[0].id = cudaLaunchAttributePriority;
+    at[0].val.priority = side->prio;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributePriority;
-    at[0].val.priority = side->prio;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = nat;
     cudaLaunchKernelEx(&cfg, k, args...);
+}
+
+template <class... A>
+inline void side_launch_on(cudaStream_t st, void (*k)(A...), dim3 grid, int threads, const SideStream* side,
+                           A... args)
+{
+    cudaLaunchAttribute at[1];
+    side_launch_with(at, 1, st, k, grid, threads, side, args...);
 }
 
 template <class... A>
 inline void side_launch(void (*k)(A...), dim3 grid, int threads, const SideStream* side, A... args)
 {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(threads);
-    cfg.stream = side->s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributePriority;
-    at[0].val.priority = side->prio;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k, args...);
+    side_launch_on(side->s, k, grid, threads, side, args...);
 }
+
+// The same for a kernel that may start beside the end of the kernel before it
+// in the stream, which calls release_next_grid; it calls wait_for_prior_grid.
+template <class... A>
+inline void side_launch_early(void (*k)(A...), dim3 grid, int threads, const SideStream* side, A... args)
+{
+    cudaLaunchAttribute at[2];
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    side_launch_with(at, 2, side->s, k, grid, threads, side, args...);
+}
+
+// Blocks of kz_scalars (at most one on each of the 152 SMs) up to which
+// k_cover_apply is launched early.
+constexpr unsigned kEarlyCoverBlocks = 152;
 
 template <class C>
 struct Ops {
@@ -117,13 +112,23 @@ struct Ops {
             cudaEventRecord(side->bnd_done, side->s);
             kz_fused<C><<<g.zgrid, kZThreads, kFusedSmem, s>>>(P, D);
             cudaEventRecord(side->collide_done, s);
-            cudaStreamWaitEvent(side->s, side->collide_done, 0);
-            side_launch(k_scalars_particles<C>, pg1, kPartThreads, side, P, D);
-            cudaStreamWaitEvent(side->s, side->mark_done, 0);
             // covering touches only nodes next to particles, whose fields the
             // side-stream kernels wrote, and leaves the next step's uniform
-            // correction in the other buffer: it runs beside the transport
-            side_launch(k_cover_apply<C>, pg2, kCoverThreads, side, P, D);
+            // correction in the other buffer: it runs beside the transport.
+            // Where the transport leaves room on every SM it starts beside
+            // k_scalars_particles (24^3 FP32: 56.1 -> 51.8 us a step); its
+            // waiting blocks would hold up a transport that fills the chip
+            // (96^3 FP64: 1351 -> 1417 us)
+            const bool early = g.zgrid_s.x * g.zgrid_s.y * g.zgrid_s.z <= kEarlyCoverBlocks;
+            if (early) cudaStreamWaitEvent(side->s, side->mark_done, 0);
+            cudaStreamWaitEvent(side->s, side->collide_done, 0);
+            side_launch(k_scalars_particles<C>, pg1, kPartThreads, side, P, D);
+            if (early) {
+                side_launch_early(k_cover_apply<C>, pg2, kCoverThreads, side, P, D);
+            } else {
+                cudaStreamWaitEvent(side->s, side->mark_done, 0);
+                side_launch(k_cover_apply<C>, pg2, kCoverThreads, side, P, D);
+            }
             cudaEventRecord(side->scal_done, side->s);
             cudaStreamWaitEvent(s, side->bnd_done, 0);
             kz_scalars<C><<<g.zgrid_s, kZThreads, kZScalSmem, s>>>(P, D);

@@ -879,6 +879,7 @@ __global__ void __launch_bounds__(kPartThreads, part_blocks_per_sm<C>()) k_scala
                                                                      const __grid_constant__ DevPtrs D)
 {
     __shared__ NodeList<C> list;
+    release_next_grid();   // k_cover_apply reads masks and positions beside this kernel
     scalars_particles_block<C>(P, D, blockIdx.y, blockIdx.x, gridDim.x, list);
 }
 
