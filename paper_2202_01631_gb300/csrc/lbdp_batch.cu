@@ -282,6 +282,8 @@ int capture_graph(lbb_batch* b, int p0)
 }  // namespace
 
 namespace lbdp {
+const SideStream* batch_side(const lbb_batch* b) { return &b->side; }
+
 void batch_release(lb_handle* h)
 {
     lbb_batch* b = h->batch;
@@ -736,11 +738,8 @@ int lbs_pump(lbs_server* s, double now, int* active, int* queued)
         for (int k = 0; k < L.q.r.n_particles && st == LB_OK; ++k)
             st = lb_add_particle(L.h, &L.q.r.particles[k], nullptr);
         if (st == LB_OK) st = lbb_set_steps(s->batch, L.h, L.q.r.steps);
-        L.q.psi.clear();
-        L.q.psi.shrink_to_fit();
-        L.q.phi.clear();
-        L.q.phi.shrink_to_fit();
         if (st != LB_OK) {
+            cudaStreamSynchronize(L.h ? L.h->stream : nullptr);   // the initial fields may still be read
             finish(s, L, st, clock());
             continue;
         }
@@ -760,6 +759,11 @@ int lbs_pump(lbs_server* s, double now, int* active, int* queued)
             cudaError_t e = cudaStreamSynchronize(s->live.front().h->stream);
             if (e != cudaSuccess) st = LB_ERR_CUDA;
         }
+    }
+    // the initial fields have been read
+    for (Live& L : s->live) {
+        std::vector<double>().swap(L.q.psi);
+        std::vector<double>().swap(L.q.phi);
     }
     // retire the boxes that have run all their steps
     for (size_t i = 0; i < s->live.size();) {

@@ -101,8 +101,10 @@ extern const BatchOps kBatchF16;
 extern const BatchOps kBatchBF16;
 
 cudaError_t launch_bflag(const DevParams& P, const uint8_t* mask, uint8_t* bflag, cudaStream_t s);
-cudaError_t launch_claim(const DevParams& P, uint8_t* m0, uint8_t* m1, const DevPart* parts, int p,
-                         unsigned long long* count, cudaStream_t s);
+// particle p of a box: its record q to the device, its nodes claimed in both
+// masks and taken off the fluid node count
+cudaError_t launch_claim(const DevParams& P, uint8_t* m0, uint8_t* m1, DevPart* parts, int p, const DevPart& q,
+                         long long* nfluid, cudaStream_t s);
 
 // Placement of a handle's device state: one region from cudaMalloc, or from
 // the arena of the batch that owns the handle.
@@ -111,6 +113,9 @@ DevPtrs handle_ptrs(const lb_handle* h, int src);
 int lb_create_in(const lb_params* p, lbb_batch* batch, void* region, lb_handle** out);
 // Return a member box's region to its batch and drop it from the batch.
 void batch_release(lb_handle* h);
+// The side streams of the batch, which a member box that steps by itself uses
+// too: its work goes to the batch's stream.
+const SideStream* batch_side(const lbb_batch* b);
 
 }  // namespace lbdp
 
@@ -124,7 +129,7 @@ struct lb_handle {
     int device;
     int cur;   // which buffer of each pair holds the current state
     lbb_batch* batch;   // owning batch, or NULL for a standalone box
-    lbdp::SideStream side;   // particle kernels' stream (side.s NULL until created)
+    lbdp::SideStream side;   // particle kernels' streams (a batch member has none of its own)
     void* region;       // the single device allocation holding every array below
     size_t region_bytes;
     void* f[2];
@@ -148,7 +153,6 @@ struct lb_handle {
     double* staging;   // 6N FP64 for host transfers: rho, u[3], psi, phi
     double* red_part;
     double* red_out;
-    unsigned long long* count;
     int red_blocks;
     int zplanes[2];   // z chunk length of kz_fused, kz_scalars (0 = size heuristic)
     // lb_step's CUDA graphs of kGraphSteps steps from parity 0 / 1, and the

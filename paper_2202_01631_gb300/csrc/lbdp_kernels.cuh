@@ -1460,21 +1460,32 @@ static __global__ void k_sums_final(const double* part, int nblocks, double* out
     for (int k = 0; k < 3; ++k) out[k] = s[k];
 }
 
-// New sphere: claim the fluid nodes strictly inside it (both mask buffers)
-// and count them.
-static __global__ void k_claim(DevParams P, uint8_t* m0, uint8_t* m1, const DevPart* parts, int p,
-                               unsigned long long* count)
+// New sphere q as particle p: its record, and the fluid nodes strictly inside it
+// claimed in both mask buffers and taken off the fluid node count.
+static __global__ void k_claim(DevParams P, uint8_t* m0, uint8_t* m1, DevPart* parts, int p,
+                               const __grid_constant__ DevPart q, long long* nfluid)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) parts[p] = q;
     const size_t N = (size_t)P.N;
+    int claimed = 0;
     for (size_t n = blockIdx.x * (size_t)blockDim.x + threadIdx.x; n < N; n += (size_t)gridDim.x * blockDim.x) {
         if (m0[n]) continue;
         const int x = (int)(n % P.nx), y = (int)((n / P.nx) % P.ny), z = (int)(n / ((size_t)P.nx * P.ny));
-        if (inside_sphere(P, parts[p], x, y, z)) {
+        if (inside_sphere(P, q, x, y, z)) {
             m0[n] = (uint8_t)(p + 1);
             m1[n] = (uint8_t)(p + 1);
-            atomicAdd(count, 1ull);
+            ++claimed;
         }
     }
+    if (claimed) atomicAdd((unsigned long long*)nfluid, (unsigned long long)(-(long long)claimed));
+}
+
+// Staging of a new box: rho0 at every node, and the fluid node count.
+static __global__ void k_rest(double* rho, double rho0, long long N, long long* nfluid)
+{
+    if (blockIdx.x == 0 && threadIdx.x == 0) *nfluid = N;
+    for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N; n += (long long)gridDim.x * blockDim.x)
+        rho[n] = rho0;
 }
 
 // Boundary flags of every node from a mask: fluid node with a solid neighbour.
