@@ -676,22 +676,22 @@ __device__ __forceinline__ void fdiv_compute(const DevParams& P, const DevPtrs& 
 // then renormalise.  For |w| < 0.1 both ratios are their Taylor series in
 // |w|^2, exact to double precision with six terms; the renormalisation is one
 // Newton step of 1/sqrt around 1 (|m'| = 1 up to rounding).
-__device__ __forceinline__ void rotate_unit(const double m[3], const double w[3], double out[3])
+// By one warp (all lanes call it): lanes 0, 1 and 2 hold the components of m, w
+// and the result, and one evaluates each series.
+__device__ __forceinline__ double rotate_unit(const double (&m)[3], const double (&w)[3], int lane)
 {
     const double w2 = dot_x(w[0], w[1], w[2], w[0], w[1], w[2]);
     double s1, c1, cw;
     if (w2 < 0.01) {
         // products with the rounded reciprocals: the divisions would be ten
-        // dependent chains on the FP64 pipe
-        s1 = fma_x(-w2 * (1.0 / 6.0),
-                   fma_x(-w2 * (1.0 / 20.0),
-                         fma_x(-w2 * (1.0 / 42.0),
-                               fma_x(-w2 * (1.0 / 72.0), fma_x(-w2 * (1.0 / 110.0), 1.0, 1.0), 1.0), 1.0), 1.0), 1.0);
-        c1 = 0.5 * fma_x(-w2 * (1.0 / 12.0),
-                         fma_x(-w2 * (1.0 / 30.0),
-                               fma_x(-w2 * (1.0 / 56.0),
-                                     fma_x(-w2 * (1.0 / 90.0), fma_x(-w2 * (1.0 / 132.0), 1.0, 1.0), 1.0), 1.0), 1.0),
-                         1.0);
+        // dependent chains on the FP64 pipe.  Lane 0: s1, others: 2 c1
+        const bool s = lane == 0;
+        const double k0 = s ? 1.0 / 6.0 : 1.0 / 12.0, k1 = s ? 1.0 / 20.0 : 1.0 / 30.0, k2 = s ? 1.0 / 42.0 : 1.0 / 56.0,
+                     k3 = s ? 1.0 / 72.0 : 1.0 / 90.0, k4 = s ? 1.0 / 110.0 : 1.0 / 132.0;
+        const double t =
+            fma_x(-w2 * k0, fma_x(-w2 * k1, fma_x(-w2 * k2, fma_x(-w2 * k3, fma_x(-w2 * k4, 1.0, 1.0), 1.0), 1.0), 1.0), 1.0);
+        s1 = __shfl_sync(0xffffffffu, t, 0);
+        c1 = 0.5 * __shfl_sync(0xffffffffu, t, 1);
         cw = fma_x(-w2, c1, 1.0);
     } else {
         const double wn = sqrt(w2);
@@ -699,136 +699,138 @@ __device__ __forceinline__ void rotate_unit(const double m[3], const double w[3]
         cw = cos(wn);
         c1 = (1.0 - cw) / w2;
     }
-    const double wxm[3] = {cross_x(w[1], m[2], w[2], m[1]), cross_x(w[2], m[0], w[0], m[2]),
-                           cross_x(w[0], m[1], w[1], m[0])};
+    const int a = lane < 3 ? lane : 0, a1 = a == 2 ? 0 : a + 1, a2 = a == 0 ? 2 : a - 1;
+    auto at = [](const double (&v)[3], int k) { return k == 0 ? v[0] : k == 1 ? v[1] : v[2]; };
+    const double wxm = cross_x(at(w, a1), at(m, a2), at(w, a2), at(m, a1));
     const double wm = mul_x(dot_x(w[0], w[1], w[2], m[0], m[1], m[2]), c1);
-    double r[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) r[a] = fma_x(w[a], wm, fma_x(wxm[a], s1, mul_x(m[a], cw)));
-    const double nn2 = dot_x(r[0], r[1], r[2], r[0], r[1], r[2]);
-    const double sc = fma_x(-0.5, nn2, 1.5);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) out[a] = mul_x(r[a], sc);
+    const double r = fma_x(at(w, a), wm, fma_x(wxm, s1, mul_x(at(m, a), cw)));
+    const double r0 = __shfl_sync(0xffffffffu, r, 0), r1 = __shfl_sync(0xffffffffu, r, 1), r2 = __shfl_sync(0xffffffffu, r, 2);
+    const double nn2 = dot_x(r0, r1, r2, r0, r1, r2);
+    return mul_x(r, fma_x(-0.5, nn2, 1.5));
 }
 
-// Implicit particle update of particle p by warp 0 of the last block, from
-// the link totals tot[0..26] (F0[3], T0[3], zeta upper triangle):
+// Implicit particle update of particle p by the whole last block (at least
+// four warps), from the link totals tot[0..5] (F0[3], T0[3]), the upper
+// triangle z[21] of zeta and the surface fluxes tot[kLinkGpsi...]:
 //   (Mdiag + zeta) V(t+1) = Mdiag V(t) + [F0 + impulses + loads; T0 + ...]
-// (symmetric positive definite: Cholesky with lane a holding row a), force
-// and torque F0 - zeta V, then the position and orientation after the step.
-// FP64 throughout; the work is spread over lanes because GB300 issues FP64
-// at a low rate.  Ls is scratch for 36 doubles.
+// (symmetric positive definite), force and torque F0 - zeta V, then the
+// position and orientation after the step.  FP64 throughout.  A warp issues one
+// FP64 instruction in 64 cycles whether it depends on the one before or not, so
+// what counts is the longest instruction stream of a warp: a thread per element
+// of the matrix, eliminated above and below the pivot at once (a reciprocal, a
+// product and an update per pivot, no substitution afterwards), then the rest
+// shared by four warps.  By Cholesky in one warp with everything after it in
+// lanes of that warp it took 16 thousand cycles of k_links, 25 thousand with a
+// spinning sphere; so 9 and 13 thousand (24^3 FP32: 54 -> 48 us a step, with the
+// block sums loaded eight at a time).
+// G is scratch for 48 doubles.
 static __device__ __noinline__ void particle_update(int3 L3, int3 per3, DevPart* parts, unsigned* ticket, int* err, int p,
-                                             const DevPart& q, const double* tot, double* Ls)
+                                             const DevPart& q, const double* tot, const double* z, double* G)
 {
-    const int lane = threadIdx.x & 31;
-    const unsigned full = 0xffffffffu;
-    if (lane == 0) ticket[p] = 0u;
-    const int a = lane < 6 ? lane : 5;   // lanes >= 6 shadow row 5
-    double zrow[6];
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double* V = G + 42;   // velocity and spin after the step
+    // element (a, c) of [Mdiag + zeta | b] at G[7 a + c]
+    auto zeta = [&](int a, int c) {
         const int lo = min(a, c), hi = max(a, c);
-        zrow[c] = tot[6 + lo * 6 - (lo * (lo - 1)) / 2 + (hi - lo)];
-    }
-    const double Ma = a < 3 ? q.M : q.I;
-    const double F0a = a < 3 ? add_x(add_x(tot[a], q.imp_f[a]), q.ext_f[a])
-                             : add_x(add_x(tot[a], q.imp_t[a - 3]), q.ext_t[a - 3]);
-    double xv[6];
-#pragma unroll
-    for (int c = 0; c < 6; ++c) xv[c] = c < 3 ? q.U[c] : q.W[c - 3];
-    if (!q.fixed) {
-        double Arow[6];
-#pragma unroll
-        for (int c = 0; c < 6; ++c) Arow[c] = c == a ? add_x(zrow[c], Ma) : zrow[c];
-        const double ba = fma_x(Ma, a < 3 ? q.U[a] : q.W[a - 3], F0a);
-        // right-looking Cholesky A = L L^T: at step j lane j holds the pivot
-        double rs[6];
+        return z[lo * 6 - (lo * (lo - 1)) / 2 + (hi - lo)];
+    };
+    auto load = [&](int a) {   // F0 + impulses + loads
+        return a < 3 ? add_x(add_x(tot[a], q.imp_f[a]), q.ext_f[a])
+                     : add_x(add_x(tot[a], q.imp_t[a - 3]), q.ext_t[a - 3]);
+    };
+    auto vel = [&](int a) { return a < 3 ? q.U[a] : q.W[a - 3]; };
+    if (q.fixed) {
+        if (threadIdx.x < 6) V[threadIdx.x] = vel(threadIdx.x);
+    } else {
+        const int e = threadIdx.x, a = e / 7, c = e % 7;
+        const bool mine = e < 42;
+        double x = 0.0;
+        if (mine) {
+            const double M = a < 3 ? q.M : q.I;
+            x = c == 6 ? fma_x(M, vel(a), load(a)) : a == c ? add_x(zeta(a, c), M) : zeta(a, c);
+            G[e] = x;
+        }
+        __syncthreads();
         bool ok = true;
-#pragma unroll
+        double ra = 0.0;   // reciprocal of the pivot of row a
+#pragma unroll 1
         for (int j = 0; j < 6; ++j) {
-            const double piv = __shfl_sync(full, Arow[j], j);
-            ok = ok && (piv > 0.0);
-            rs[j] = rsqrt(fmax(piv, 1e-300));
-            const double laj = mul_x(Arow[j], rs[j]);   // L[a][j] for a >= j
-            if (lane < 6) Ls[a * 6 + j] = laj;
-#pragma unroll
-            for (int c = j + 1; c < 6; ++c) Arow[c] = fma_x(-laj, __shfl_sync(full, laj, c), Arow[c]);
+            const double piv = G[8 * j];
+            double f = 0.0, g = 0.0;
+            if (mine) {
+                f = G[7 * a + j];
+                g = G[7 * j + c];
+            }
+            __syncthreads();
+            if (mine) {
+                ok = ok && (unsigned)__double2hiint(piv) - 1u < 0x7ff00000u;   // positive, not NaN
+                const double r = __drcp_rn(fmax(piv, 1e-300));
+                // the pivot row keeps its elements; columns up to j are never read again
+                if (a == j)
+                    ra = r;
+                else
+                    G[e] = x = fma_x(-mul_x(f, r), g, x);
+            }
+            __syncthreads();
         }
-        __syncwarp();
-        // L y = b, then L^T x = y (uniform in the warp; L from shared memory)
-        double yv[6];
-#pragma unroll
-        for (int j = 0; j < 6; ++j) {
-            double t = __shfl_sync(full, ba, j);
-#pragma unroll
-            for (int k = 0; k < j; ++k) t = fma_x(-Ls[j * 6 + k], yv[k], t);
-            yv[j] = mul_x(t, rs[j]);
-        }
-#pragma unroll
-        for (int j = 5; j >= 0; --j) {
-            double t = yv[j];
-#pragma unroll
-            for (int k = j + 1; k < 6; ++k) t = fma_x(-Ls[k * 6 + j], xv[k], t);
-            xv[j] = mul_x(t, rs[j]);
-        }
-        if (!ok && lane == 0) atomicOr(err, kErrSolve);
+        if (mine && c == 6) V[a] = mul_x(x, ra);
+        if (!ok && e == 0) atomicOr(err, kErrSolve);
     }
+    __syncthreads();
     DevPart& dp = parts[p];
-    if (lane == 0) {
+    if (warp == 0) {
+        if (lane == 0) ticket[p] = 0u;
+        if (lane < 6) {
+            double zv = 0.0;
+#pragma unroll 1
+            for (int c = 0; c < 6; ++c) zv = fma_x(zeta(lane, c), V[c], zv);
+            const double f = add_x(load(lane), -zv);
+            if (lane < 3)
+                dp.force[lane] = f;
+            else
+                dp.torque[lane - 3] = f;
+        }
+    } else if (warp == 1) {
+        if (lane < 3) {
+            const int a = lane;
+            const int L = a == 0 ? L3.x : (a == 1 ? L3.y : L3.z);
+            const int per = a == 0 ? per3.x : (a == 1 ? per3.y : per3.z);
+            const double v = V[a], w = V[3 + a];
+            dp.U[a] = v;
+            dp.W[a] = w;
+            dp.Uf[a] = (float)v;
+            dp.Wf[a] = (float)w;
+            dp.imp_f[a] = 0.0;
+            dp.imp_t[a] = 0.0;
+            double X = add_x(q.X[a], v);
+            if (per) {
+                if (X >= L)
+                    X -= L;
+                else if (X < 0.0)
+                    X += L;
+            } else if (X - q.R < 1.0 || X + q.R > L - 2.0) {
+                atomicOr(err, kErrWall);
+            }
+            dp.Xn[a] = X;
+            const double f = floor(X);
+            const double fr = X - f;
+            dp.gn.Xi[a] = (int)f;
+            dp.gn.frd[a] = fr;
+            dp.gn.fr[a] = (float)fr;
+            dp.gn.fl[a] = (fr > 0.0 ? kFrPos : 0) | (fr < 0.5 ? kFrBelowHalf : 0) | (fr > 0.5 ? kFrAboveHalf : 0);
+        }
+    } else if (warp == 2) {
+        const double w3[3] = {V[3], V[4], V[5]}, m[3] = {q.m[0], q.m[1], q.m[2]};
+        double mn = lane == 0 ? m[0] : lane == 1 ? m[1] : m[2];
+        if (w3[0] != 0.0 || w3[1] != 0.0 || w3[2] != 0.0) mn = rotate_unit(m, w3, lane);   // uniform in the warp
+        if (lane < 3) dp.mn[lane] = mn;
+    } else if (warp == 3 && lane < 2) {
         // psi, phi carried into the surface: sum 6 w g c.u_b with u_b at V(t+1)
-        double wps = tot[kLinkGpsi + 6], wph = tot[kLinkGphi + 6];
-#pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            wps = fma_x(tot[kLinkGpsi + c], xv[c], wps);
-            wph = fma_x(tot[kLinkGphi + c], xv[c], wph);
-        }
-        dp.wall_psi = wps;
-        dp.wall_phi = wph;
-    }
-    if (lane < 6) {
-        double zv = 0.0;
-#pragma unroll
-        for (int c = 0; c < 6; ++c) zv = fma_x(zrow[c], xv[c], zv);
-        if (a < 3)
-            dp.force[a] = add_x(F0a, -zv);
-        else
-            dp.torque[a - 3] = add_x(F0a, -zv);
-    }
-    if (lane < 3) {
-        const int L = a == 0 ? L3.x : (a == 1 ? L3.y : L3.z);
-        const int per = a == 0 ? per3.x : (a == 1 ? per3.y : per3.z);
-        const double v = a == 0 ? xv[0] : (a == 1 ? xv[1] : xv[2]);
-        const double w = a == 0 ? xv[3] : (a == 1 ? xv[4] : xv[5]);
-        dp.U[a] = v;
-        dp.W[a] = w;
-        dp.Uf[a] = (float)v;
-        dp.Wf[a] = (float)w;
-        dp.imp_f[a] = 0.0;
-        dp.imp_t[a] = 0.0;
-        double X = add_x(q.X[a], v);
-        if (per) {
-            if (X >= L)
-                X -= L;
-            else if (X < 0.0)
-                X += L;
-        } else if (X - q.R < 1.0 || X + q.R > L - 2.0) {
-            atomicOr(err, kErrWall);
-        }
-        dp.Xn[a] = X;
-        const double f = floor(X);
-        const double fr = X - f;
-        dp.gn.Xi[a] = (int)f;
-        dp.gn.frd[a] = fr;
-        dp.gn.fr[a] = (float)fr;
-        dp.gn.fl[a] = (fr > 0.0 ? kFrPos : 0) | (fr < 0.5 ? kFrBelowHalf : 0) | (fr > 0.5 ? kFrAboveHalf : 0);
-    }
-    if (lane == 0) {
-        const double w3[3] = {xv[3], xv[4], xv[5]};
-        double mn[3] = {q.m[0], q.m[1], q.m[2]};
-        if (w3[0] != 0.0 || w3[1] != 0.0 || w3[2] != 0.0) rotate_unit(q.m, w3, mn);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) dp.mn[c] = mn[c];
+        const double* g = tot + (lane == 0 ? kLinkGpsi : kLinkGphi);
+        double s = g[6];
+#pragma unroll 1
+        for (int c = 0; c < 6; ++c) s = fma_x(g[c], V[c], s);
+        (lane == 0 ? dp.wall_psi : dp.wall_phi) = s;
     }
 }
 

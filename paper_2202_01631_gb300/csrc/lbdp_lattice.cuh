@@ -199,7 +199,7 @@ enum : int {
 // sum 6 w psi (c, r x c) [6], sum 6 w psi c.v_s, and the same for phi
 constexpr int kLinkK = 41;
 constexpr int kLinkGpsi = 27, kLinkGphi = 34;
-static_assert(kLinkK <= 64, "the particle update keeps its scratch at smem + 64");
+static_assert(kLinkK <= 64, "room for the totals in shared memory");
 constexpr int kCoverK = 9;    // per-block cover partials: impulse F[3], T[3], dpsi, dphi,
                               // dcount
 constexpr int kMaxPartBlocks = 128;

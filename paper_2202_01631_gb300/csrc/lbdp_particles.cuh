@@ -363,8 +363,8 @@ __global__ void __launch_bounds__(kPartThreads) k_f_part(const __grid_constant__
 // blocks of a particle split its link box; the last block of the particle (a
 // ticket counter) sums the partials in block order and solves
 //   (Mdiag + zeta) V(t+1) = Mdiag V(t) + [F0; T0]
-// (symmetric positive definite: Cholesky), then stores the new velocity and
-// the position/orientation after the step.
+// (symmetric positive definite), then stores the new velocity and the
+// position/orientation after the step.
 //
 // With a = 36 w_i (2 on axis links, 1 on diagonal ones), c = c_i, r = x - X and
 // D = r + fr the node's integer offset from floor(X), the sums over a node's
@@ -400,7 +400,7 @@ struct LinkSmem {
     int ri[kRowNodes][kRowI];
     double col[kRowGroups][kRow];
     double red[kPartThreads];
-    double tot[64 + 36];   // link totals, scratch of the particle update
+    double tot[64];        // link totals
     bool last;
 };
 
@@ -662,9 +662,17 @@ __device__ __forceinline__ void links_block(const DevParams& P, const DevPtrs& D
         const int k = threadIdx.x % K, g = threadIdx.x / K;
         double s = 0.0;
         if (g < G) {
+            // eight loads in flight (a loop of one at a time is a chain of L2
+            // accesses: 10 of 54 thousand cycles with 42 blocks)
             const double* pb = D.link_part + (size_t)p * kMaxPartBlocks * K + k;
-#pragma unroll 4
-            for (int b = g; b < nbi; b += G) s += __ldcg(pb + (size_t)b * K);
+            for (int b0 = g; b0 < nbi; b0 += 8 * G) {
+                double v[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = b0 + j * G < nbi ? __ldcg(pb + (size_t)(b0 + j * G) * K) : 0.0;
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (b0 + j * G < nbi) s += v[j];
+            }
         }
         if (g < G) sm.red[g * K + k] = s;
         __syncthreads();
@@ -676,21 +684,19 @@ __device__ __forceinline__ void links_block(const DevParams& P, const DevPtrs& D
         }
         __syncthreads();
     }
-    double z = 0.0;
-    if (threadIdx.x >= 6 && threadIdx.x < 27) {
-        int a = 0, k = threadIdx.x - 6;
-        while (k >= 6 - a) {
-            k -= 6 - a;
-            ++a;
+    {   // red is free again: zeta goes there, its three blocks on a warp each
+        const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+        if (w < 3 && l < (w == 1 ? 9 : 6)) {
+            const int i = w == 1 ? l / 3 : l < 3 ? 0 : l < 5 ? 1 : 2;   // row and column in the block
+            const int j = w == 1 ? l % 3 : l < 3 ? l : l < 5 ? l - 2 : 2;
+            const int a = w == 2 ? i + 3 : i, b = w == 0 ? j : j + 3;
+            sm.red[a * 6 - (a * (a - 1)) / 2 + (b - a)] =
+                zeta_entry(a, b, sm.tot + 6, q.g.frd, prm<double>(P).rho0 / 6.0);
         }
-        z = zeta_entry(a, a + k, sm.tot + 6, q.g.frd, prm<double>(P).rho0 / 6.0);
     }
     __syncthreads();
-    if (threadIdx.x >= 6 && threadIdx.x < 27) sm.tot[threadIdx.x] = z;
-    __syncthreads();
-    if (threadIdx.x >= 32) return;
     particle_update(make_int3(P.nx, P.ny, P.nz), make_int3(P.per[0], P.per[1], P.per[2]), D.parts, D.link_ticket,
-                    D.err, p, q, sm.tot, sm.tot + 64);   // totals in tot[0..K-1], K <= 64
+                    D.err, p, q, sm.tot, sm.red, sm.red + 32);   // totals in tot[0..K-1]
 }
 
 template <class C>
