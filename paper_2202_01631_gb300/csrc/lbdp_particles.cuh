@@ -383,13 +383,21 @@ __global__ void __launch_bounds__(kPartThreads) k_f_part(const __grid_constant__
 //     sum 6 w (c, r x c) = (B, r x B)/6 and sum 6 w c.v_s (finite differences),
 //     or the same with weight 1 on the six D3Q7 links (lattice Boltzmann).
 // So a link costs its slip velocity and nothing else.  Each node's values are
-// one row of 20 numbers of the arithmetic precision and 27 integers; a thread
-// per column adds the rows in FP64 and int64.
-// Measured on GB300, FP32, one sphere R = 8: 56 us with 41 FP64 sums over the
-// links (250 registers, 84 KB of shared memory).
+// one row of 26 numbers of the arithmetic precision and 27 integers; a thread
+// per column and quarter of the rows adds them in FP64 and int64.  Two threads
+// of different warps share a node, one for its stress and the force of it
+// (columns 20 to 25), one for the rest: a block has fewer nodes than threads,
+// and what bounds it is the length of one thread's work.
+// Measured on GB300: FP32, one sphere R = 8, 56 us with 41 FP64 sums over the
+// links (250 registers, 84 KB of shared memory), 33 with the rows; the rows'
+// part of the block 16.5 thousand cycles with a thread per node, 10.0 with two
+// (24^3; FP64 32^3 100 and 70), the kernels before the bulk 54.3 -> 48.6 us at
+// 24^3, 160 -> 144 in FP64 at 32^3 (with the shared particle update).
 // ---------------------------------------------------------------------------
-constexpr int kRowF = 20, kRowI = 27, kRow = kRowF + kRowI, kRowGroups = 2, kRowNodes = 64;
-static_assert(kRowGroups * kRow <= kPartThreads, "a thread per column and group of rows");
+constexpr int kRowP = 20, kRowF = kRowP + 6, kRowI = 27, kRow = kRowF + kRowI, kRowGroups = 4;
+constexpr int kRowNodes = kPartThreads / 2;   // nodes of a round: two threads each
+static_assert(kRowGroups * kRowF <= kPartThreads && kRowGroups * kRowI <= kPartThreads,
+              "a thread per column and group of rows");
 
 template <class C>
 struct LinkSmem {
@@ -404,7 +412,80 @@ struct LinkSmem {
     bool last;
 };
 
-// Node n of the link box of particle q (in shared memory): its row.
+// Integer sums of the links in bits: A = sum a c c^T (xx yy zz xy xz yz), B =
+// sum a c.
+__device__ __forceinline__ void link_ints(unsigned bits, int (&A)[6], int (&B)[3])
+{
+#pragma unroll
+    for (int k = 0; k < 6; ++k) A[k] = 0;
+    B[0] = B[1] = B[2] = 0;
+#pragma unroll
+    for (int i = 1; i < 19; ++i) {
+        const int k = (int)(bits >> i & 1u) * (i < 7 ? 2 : 1);
+        A[0] += k * cx(i) * cx(i);
+        A[1] += k * cy(i) * cy(i);
+        A[2] += k * cz(i) * cz(i);
+        A[3] += k * cx(i) * cy(i);
+        A[4] += k * cx(i) * cz(i);
+        A[5] += k * cy(i) * cz(i);
+        B[0] += k * cx(i);
+        B[1] += k * cy(i);
+        B[2] += k * cz(i);
+    }
+}
+
+// Node n of the link box of particle q (in shared memory): the force of its
+// stress (the one the fluid's force uses this step, k_pt_part) on the links and
+// its torque, columns kRowP to kRowP + 5 of the row.
+template <class C>
+__device__ __forceinline__ void link_stress(const DevParams& P, const DevPtrs& D, const DevPart& q, int p, int n,
+                                            typename C::real (&rf)[kRowF + 1])
+{
+    using R = typename C::real;
+    using F = typename C::fld_t;
+    const PrmR<R>& Q = prm<R>(P);
+    if (!P.thermo) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) rf[kRowP + k] = 0;
+        return;
+    }
+    int x, y, z;
+    node_coords(P, n, x, y, z);
+    Around a;
+    look_around(P, D, x, y, z, a);
+    GAcc<F, 2> ga;
+#pragma unroll
+    for (int i = 0; i < 19; ++i) ga.nb[i] = a.nb[i];
+    ga.n = n;
+    ga.mk = D.mask;
+    ga.f[0] = (const F*)D.psi_src;
+    ga.f[1] = (const F*)D.phi_src;
+    R m1, m2, pt[kPtFields];
+    mup_values<C>(P, D, x, y, z, ga, corr_r<R>(D, 0), corr_r<R>(D, 1), m1, m2, pt);
+#pragma unroll
+    for (int k = 0; k < kPtFields; ++k) pt[k] = (R)(F)pt[k];
+    int A[6], B[3];
+    link_ints(links_into(a, p + 1), A, B);
+    const R Bf[3] = {(R)B[0], (R)B[1], (R)B[2]};
+    const R gB = mul_x(Q.kappa, dot_x(pt[1], pt[2], pt[3], Bf[0], Bf[1], Bf[2]));
+    R m[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) m[k] = mul_x((R)(1.0 / 6.0), fma_x(gB, pt[1 + k], mul_x(pt[0], Bf[k])));
+    NodeLinks<R> l;
+    node_links<R>(P, q, x, y, z, l);
+    const R Af[6] = {(R)A[0], (R)A[1], (R)A[2], (R)A[3], (R)A[4], (R)A[5]};
+    const R Ag[3] = {dot_x(Af[0], Af[3], Af[4], pt[1], pt[2], pt[3]), dot_x(Af[3], Af[1], Af[5], pt[1], pt[2], pt[3]),
+                     dot_x(Af[4], Af[5], Af[2], pt[1], pt[2], pt[3])};
+    const R k = mul_x(Q.kappa, (R)(1.0 / 12.0));
+    rf[kRowP] = m[0];
+    rf[kRowP + 1] = m[1];
+    rf[kRowP + 2] = m[2];
+    rf[kRowP + 3] = fma_x(k, cross_x(Ag[1], pt[3], Ag[2], pt[2]), cross_x(l.r0[1], m[2], l.r0[2], m[1]));
+    rf[kRowP + 4] = fma_x(k, cross_x(Ag[2], pt[1], Ag[0], pt[3]), cross_x(l.r0[2], m[0], l.r0[0], m[2]));
+    rf[kRowP + 5] = fma_x(k, cross_x(Ag[0], pt[2], Ag[1], pt[1]), cross_x(l.r0[0], m[1], l.r0[1], m[0]));
+}
+
+// Node n of the link box of particle q (in shared memory): the rest of its row.
 template <class C>
 __device__ __forceinline__ void link_row(const DevParams& P, const DevPtrs& D, const DevPart& q, int p, int n,
                                          typename C::real (&rf)[kRowF + 1], int (&ri)[kRowI])
@@ -430,21 +511,6 @@ __device__ __forceinline__ void link_row(const DevParams& P, const DevPtrs& D, c
     const R ps = (R)((const F*)D.psi_src)[n] + dps, ph = (R)phi[n] + dph;
     R gphi[3];
     grad_phi_around<R, F>(a, phi, n, ph, dph, gphi);
-    R pt[kPtFields] = {0, 0, 0, 0};
-    if (P.thermo) {
-        // the stress the fluid's force uses this step (k_pt_part)
-        GAcc<F, 2> ga;
-#pragma unroll
-        for (int i = 0; i < 19; ++i) ga.nb[i] = a.nb[i];
-        ga.n = n;
-        ga.mk = D.mask;
-        ga.f[0] = (const F*)D.psi_src;
-        ga.f[1] = phi;
-        R m1, m2;
-        mup_values<C>(P, D, x, y, z, ga, dps, dph, m1, m2, pt);
-#pragma unroll
-        for (int k = 0; k < kPtFields; ++k) pt[k] = (R)(F)pt[k];
-    }
     // bounced populations, 2 sum c g_i
     R m[3] = {0, 0, 0};
 #pragma unroll
@@ -473,45 +539,18 @@ __device__ __forceinline__ void link_row(const DevParams& P, const DevPtrs& D, c
             slip = fma_x(P.scheme ? (i < 7 ? (R)1 : (R)0) : w6, cvs, slip);
         }
     }
-    // integer sums of the links
-    int A[6] = {0, 0, 0, 0, 0, 0}, B[3] = {0, 0, 0}, B7[3] = {0, 0, 0};   // A: xx yy zz xy xz yz
+    int A[6], B[3], B7[3] = {0, 0, 0};
+    link_ints(bits, A, B);
 #pragma unroll
-    for (int i = 1; i < 19; ++i) {
-        const int k = (int)(bits >> i & 1u) * (i < 7 ? 2 : 1);
-        A[0] += k * cx(i) * cx(i);
-        A[1] += k * cy(i) * cy(i);
-        A[2] += k * cz(i) * cz(i);
-        A[3] += k * cx(i) * cy(i);
-        A[4] += k * cx(i) * cz(i);
-        A[5] += k * cy(i) * cz(i);
-        B[0] += k * cx(i);
-        B[1] += k * cy(i);
-        B[2] += k * cz(i);
-        if (i < 7) {
-            const int one = (int)(bits >> i & 1u);
-            B7[0] += one * cx(i);
-            B7[1] += one * cy(i);
-            B7[2] += one * cz(i);
-        }
+    for (int i = 1; i < 7; ++i) {
+        const int one = (int)(bits >> i & 1u);
+        B7[0] += one * cx(i);
+        B7[1] += one * cy(i);
+        B7[2] += one * cz(i);
     }
     const R Bf[3] = {(R)B[0], (R)B[1], (R)B[2]};
-    if (P.thermo) {
-        const R gB = mul_x(Q.kappa, dot_x(pt[1], pt[2], pt[3], Bf[0], Bf[1], Bf[2]));
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-            m[k] = fma_x((R)(1.0 / 6.0), fma_x(gB, pt[1 + k], mul_x(pt[0], Bf[k])), m[k]);
-    }
-    R T[3] = {cross_x(l.r0[1], m[2], l.r0[2], m[1]), cross_x(l.r0[2], m[0], l.r0[0], m[2]),
-              cross_x(l.r0[0], m[1], l.r0[1], m[0])};
-    if (P.thermo) {
-        const R Af[6] = {(R)A[0], (R)A[1], (R)A[2], (R)A[3], (R)A[4], (R)A[5]};
-        const R Ag[3] = {dot_x(Af[0], Af[3], Af[4], pt[1], pt[2], pt[3]), dot_x(Af[3], Af[1], Af[5], pt[1], pt[2], pt[3]),
-                         dot_x(Af[4], Af[5], Af[2], pt[1], pt[2], pt[3])};
-        const R k = mul_x(Q.kappa, (R)(1.0 / 12.0));
-        T[0] = fma_x(k, cross_x(Ag[1], pt[3], Ag[2], pt[2]), T[0]);
-        T[1] = fma_x(k, cross_x(Ag[2], pt[1], Ag[0], pt[3]), T[1]);
-        T[2] = fma_x(k, cross_x(Ag[0], pt[2], Ag[1], pt[1]), T[2]);
-    }
+    const R T[3] = {cross_x(l.r0[1], m[2], l.r0[2], m[1]), cross_x(l.r0[2], m[0], l.r0[0], m[2]),
+                    cross_x(l.r0[0], m[1], l.r0[1], m[0])};
     R G[7];
     {
         const R w = P.scheme ? (R)1 : (R)(1.0 / 6.0);
@@ -605,7 +644,8 @@ __device__ __forceinline__ void links_block(const DevParams& P, const DevPtrs& D
     int o[3];
     link_box(q, o);
     const int tot = P.side1[0] * P.side1[1] * P.side1[2];
-    const int col = threadIdx.x % kRow, grp = threadIdx.x / kRow;
+    const int colf = threadIdx.x % kRowF, grpf = threadIdx.x / kRowF;
+    const int coli = threadIdx.x % kRowI, grpi = threadIdx.x / kRowI;
     double accf = 0.0;
     long long acci = 0;
     for (int r = 0; (long long)r * NodeList<C>::kScanSlots * kPartThreads * nbi < tot; ++r) {
@@ -613,19 +653,23 @@ __device__ __forceinline__ void links_block(const DevParams& P, const DevPtrs& D
                                    [&](int n, int, int, int) { return D.mask[n] == 0 && D.bflag[n] != 0; });
         for (int s0 = 0; s0 < cnt; s0 += kRowNodes) {
             const int m = min(cnt - s0, kRowNodes);
-            if ((int)threadIdx.x < m)
-                link_row<C>(P, D, q, p, sm.list.n[s0 + threadIdx.x], sm.rf[threadIdx.x], sm.ri[threadIdx.x]);
-            __syncthreads();
-            if (grp < kRowGroups) {
-                if (col < kRowF)
-                    for (int r = grp; r < m; r += kRowGroups) accf += (double)sm.rf[r][col];
+            const int e = threadIdx.x % kRowNodes;
+            if (e < m) {
+                if ((int)threadIdx.x < kRowNodes)
+                    link_row<C>(P, D, q, p, sm.list.n[s0 + e], sm.rf[e], sm.ri[e]);
                 else
-                    for (int r = grp; r < m; r += kRowGroups) acci += sm.ri[r][col - kRowF];
+                    link_stress<C>(P, D, q, p, sm.list.n[s0 + e], sm.rf[e]);
             }
+            __syncthreads();
+            if (grpf < kRowGroups)
+                for (int r = grpf; r < m; r += kRowGroups) accf += (double)sm.rf[r][colf];
+            if (grpi < kRowGroups)
+                for (int r = grpi; r < m; r += kRowGroups) acci += sm.ri[r][coli];
             __syncthreads();
         }
     }
-    if (grp < kRowGroups) sm.col[grp][col] = col < kRowF ? accf : (double)acci;
+    if (grpf < kRowGroups) sm.col[grpf][colf] = accf;
+    if (grpi < kRowGroups) sm.col[grpi][kRowF + coli] = (double)acci;
     __syncthreads();
     if (threadIdx.x < kRow) {
         double s = 0.0;
@@ -638,7 +682,7 @@ __device__ __forceinline__ void links_block(const DevParams& P, const DevPtrs& D
     if (threadIdx.x < K) {
         // F0, T0, the integer sums of zeta, then the fluxes of psi and phi
         const int k = threadIdx.x;
-        double v = k < 6 ? sm.tot[k] : (k < 27 ? sm.tot[kRowF + k - 6] : sm.tot[6 + k - 27]);
+        double v = k < 6 ? sm.tot[k] + sm.tot[kRowP + k] : (k < 27 ? sm.tot[kRowF + k - 6] : sm.tot[6 + k - 27]);
         if (k < 6) {
             const PrmR<double>& Qd = prm<double>(P);
             const double kc = (2.0 * Qd.rho0 + (P.thermo ? 1.5 * Qd.A : 0.0)) / 36.0;
