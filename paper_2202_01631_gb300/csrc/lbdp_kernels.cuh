@@ -1212,7 +1212,10 @@ __device__ __forceinline__ void cover_apply_block(const DevParams& P, const DevP
     double* part = D.cover_part + ((size_t)p * kMaxPartBlocks + bi) * K;
     const int any = __syncthreads_or(changed);
     if (any) block_sum_rows<K>(acc, smem);
-    if ((int)threadIdx.x < K) part[threadIdx.x] = any ? smem[threadIdx.x] : 0.0;
+    // a block without changes stores one +0, its node count; one with changes
+    // but as many nodes covered as uncovered stores -0 there
+    if ((int)threadIdx.x < (any ? K - 1 : 0)) part[threadIdx.x] = smem[threadIdx.x];
+    if (threadIdx.x == K - 1) part[K - 1] = !any ? 0.0 : smem[K - 1] == 0.0 ? -0.0 : smem[K - 1];
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
@@ -1231,14 +1234,18 @@ __device__ __forceinline__ void cover_apply_block(const DevParams& P, const DevP
         double s[K];
 #pragma unroll
         for (int c = 0; c < K; ++c) s[c] = 0.0;
+        // nothing changed: one load a block and no FP64 instruction (64 cycles
+        // each)
+        bool nz = false;
         for (int b = lane; b < nbi; b += 32) {
             const double* cp = D.cover_part + ((size_t)k * kMaxPartBlocks + b) * K;
+            const double d = __ldcg(cp + K - 1);
+            if (__double_as_longlong(d) == 0) continue;
+            nz = true;
 #pragma unroll
-            for (int c = 0; c < K; ++c) s[c] += __ldcg(cp + c);
+            for (int c = 0; c < K - 1; ++c) s[c] += __ldcg(cp + c);
+            s[K - 1] += d;
         }
-        bool nz = false;
-#pragma unroll
-        for (int c = 0; c < K; ++c) nz = nz || s[c] != 0.0;
         if (__any_sync(0xffffffffu, nz)) {
             for (int w = 16; w > 0; w >>= 1)
 #pragma unroll
@@ -1269,19 +1276,20 @@ __device__ __forceinline__ void cover_apply_block(const DevParams& P, const DevP
         }
     }
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    double dsum_psi = 0.0, dsum_phi = 0.0, dcnt = 0.0;
+    if (threadIdx.x >= 2) return;
+    // thread 0: psi, thread 1: phi
+    double dsum = 0.0, dcnt = 0.0;
     for (int k = 0; k < P.np; ++k) {
-        dsum_psi += smem[3 * k];
-        dsum_phi += smem[3 * k + 1];
+        dsum += smem[3 * k + threadIdx.x];
         dcnt += smem[3 * k + 2];
     }
     const long long nf = *D.nfluid + (long long)dcnt;
+    const double c = dsum / (double)nf;
+    D.corr_next[threadIdx.x] = c;
+    D.corr_f_next[threadIdx.x] = (float)c;
+    __syncwarp(3u);
+    if (threadIdx.x != 0) return;
     *D.nfluid = nf;
-    D.corr_next[0] = dsum_psi / (double)nf;
-    D.corr_next[1] = dsum_phi / (double)nf;
-    D.corr_f_next[0] = (float)D.corr_next[0];
-    D.corr_f_next[1] = (float)D.corr_next[1];
     *D.cover_ticket = 0u;
 }
 
