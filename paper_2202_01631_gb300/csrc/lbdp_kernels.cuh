@@ -48,7 +48,6 @@ using CfgF32 = Cfg<float, float, float>;
 using CfgF16 = Cfg<__half, float, float>;
 using CfgBF16 = Cfg<__nv_bfloat16, float, float>;
 
-constexpr int kRowThreads = 128;
 // Threads of the kernels next to particles and of the covering kernels, and
 // the box slots a thread of the former looks at.  About a tenth of a sphere's
 // box lies next to it: a block of 128 threads finds the nodes of a full warp or
