@@ -149,12 +149,16 @@ DevPtrs cur_ptrs(const lb_handle* h)
 // run at a time, one alone on its SM in about 0.7 of the time; and the grid
 // ends with its slowest blocks, those beside a sphere above all.  FP64 (halves
 // = 1): the FP64 pipe of an SM is the limit, so the cost is the planes of the
-// blocks an SM gets, plus 1.3 per block for the recomputed halo planes.
+// blocks an SM gets, two at a time (a last one alone leaves the pipe idle at its
+// barriers and takes 1.3 of its share), plus 1.3 per block for the recomputed
+// halo planes; within 5% of the best length over ten boxes of 32^3 to 133^3
+// (without the odd block's price 16%).
 // Measured on GB300 over 1 to 128 planes (us, choice in brackets): FP32 with a
 // sphere 24^3 2 planes 31, 6 planes 44 [1]; 128^3 4 planes 123, 6 110, 8 115,
 // 12 128 [8]; 256^3 8 planes 668, 24 603, 32 597, 64 623 [32]; without one 64^3
 // 2 planes 26, 4 20, 16 31 [4]; 80 x 76 x 84 4 planes 51, 10 42, 24 57 [10];
-// FP64 32^3 1 plane 115, 6 planes 333 [1]; 96^3 4 planes 1062, 8 986, 24 1071 [8].
+// FP64 32^3 1 plane 115, 6 planes 333 [1]; 96^3 4 planes 945, 8 875, 12 861, 16
+// 1118 [12]; 102 x 107 x 95 12 planes 1439, 16 1616, 19 1383 [19].
 int default_fused_planes(const DevParams& P, int halves)
 {
     const long long cols = (long long)((P.nx + 31) / 32) * ((P.ny + 7) / 8);
@@ -169,7 +173,8 @@ int default_fused_planes(const DevParams& P, int halves)
             const double waves = blocks <= 152 ? 0.7 : blocks <= 304 ? 1.0 : blocks <= 608 ? 2.0 : (double)blocks / 304;
             cost = (waves + (P.np > 0 ? 1.5 : 0.5)) * ((p + 1) / 2 + 3);
         } else {
-            cost = ((double)((blocks + 151) / 152) + (P.np > 0 ? 0.5 : 0.25)) * (p + 1.3);
+            const long long n = (blocks + 151) / 152;
+            cost = (n % 2 ? (double)n + 0.3 : (double)n) * (p + 1.3);
         }
         if (cost < best) {
             best = cost;
