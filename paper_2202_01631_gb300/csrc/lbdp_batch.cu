@@ -739,7 +739,7 @@ int lbs_pump(lbs_server* s, double now, int* active, int* queued)
             st = lb_add_particle(L.h, &L.q.r.particles[k], nullptr);
         if (st == LB_OK) st = lbb_set_steps(s->batch, L.h, L.q.r.steps);
         if (st != LB_OK) {
-            cudaStreamSynchronize(L.h ? L.h->stream : nullptr);   // the initial fields may still be read
+            if (L.h) cudaStreamSynchronize(L.h->stream);   // the initial fields may still be read
             finish(s, L, st, clock());
             continue;
         }
@@ -755,10 +755,8 @@ int lbs_pump(lbs_server* s, double now, int* active, int* queued)
     int st = LB_OK;
     if (!s->live.empty()) {
         st = lbb_run(s->batch, (int)n, nullptr);
-        if (st == LB_OK) {
-            cudaError_t e = cudaStreamSynchronize(s->live.front().h->stream);
-            if (e != cudaSuccess) st = LB_ERR_CUDA;
-        }
+        const cudaError_t e = cudaStreamSynchronize(s->live.front().h->stream);
+        if (st == LB_OK && e != cudaSuccess) st = LB_ERR_CUDA;
     }
     // the initial fields have been read
     for (Live& L : s->live) {
