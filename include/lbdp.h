@@ -144,7 +144,9 @@ void lb_destroy(lb_handle* h);
  * second-order equilibrium of (rho, u) (Sec. "Numerical details": the system
  * starts from equilibrium).  Values at nodes inside particles are ignored.
  * A NaN or Inf in a given array (at any node) returns LB_ERR_NONFINITE and
- * leaves the box unchanged. */
+ * leaves the box unchanged.  Waits until the arrays have been copied: they may
+ * be written again on return (while the caller is capturing the handle's
+ * stream, which rules out waiting, they must live as long as its graph). */
 int lb_set_fields(lb_handle* h, const double* rho, const double* u,
                   const double* psi, const double* phi);
 

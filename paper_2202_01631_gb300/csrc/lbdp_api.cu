@@ -396,33 +396,16 @@ void lb_destroy(lb_handle* h)
 int lb_set_fields(lb_handle* h, const double* rho, const double* u, const double* psi, const double* phi)
 {
     if (!h) return LB_ERR_PARAM;
-    const size_t N = (size_t)h->dp.N;
-    // a non-finite input would spread through the whole box in a few steps:
-    // refuse it before anything is copied
-    const struct {
-        const double* a;
-        size_t n;
-    } in[4] = {{rho, N}, {u, 3 * N}, {psi, N}, {phi, N}};
-    for (const auto& v : in)
-        if (v.a)
-            for (size_t k = 0; k < v.n; ++k)
-                if (!std::isfinite(v.a[k])) return LB_ERR_NONFINITE;
-    cudaSetDevice(h->device);
-    cudaStream_t s = h->stream;
-    double* st_rho = h->staging;
-    double* st_u = h->staging + N;
-    double* st_psi = h->staging + 4 * N;
-    double* st_phi = h->staging + 5 * N;
-    if (rho) LB_TRY(cudaMemcpyAsync(st_rho, rho, N * sizeof(double), cudaMemcpyHostToDevice, s));
-    if (u) LB_TRY(cudaMemcpyAsync(st_u, u, 3 * N * sizeof(double), cudaMemcpyHostToDevice, s));
-    if (psi) LB_TRY(cudaMemcpyAsync(st_psi, psi, N * sizeof(double), cudaMemcpyHostToDevice, s));
-    if (phi) LB_TRY(cudaMemcpyAsync(st_phi, phi, N * sizeof(double), cudaMemcpyHostToDevice, s));
-    // one pass: fields from staging (or current value plus the pending uniform
-    // correction), populations to equilibrium; then the correction is spent
-    LB_TRY(h->ops->set_fields(h->dp, cur_ptrs(h), s, rho ? st_rho : nullptr, u ? st_u : nullptr,
-                              psi ? st_psi : nullptr, phi ? st_phi : nullptr));
-    LB_TRY(cudaMemsetAsync(h->corr, 0, 8 * sizeof(double), s));
-    return LB_OK;
+    const int st = queue_fields(h, rho, u, psi, phi);
+    if (st == LB_ERR_NONFINITE || !(rho || u || psi || phi)) return st;
+    // the arrays are the caller's again on return: a copy from pinned memory
+    // runs when the stream gets to it.  Under the caller's capture it is part
+    // of the caller's graph, and there is nothing to wait for
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess) cudaGetLastError();
+    if (cs != cudaStreamCaptureStatusNone) return st;
+    const int waited = cuda_status(cudaStreamSynchronize(h->stream));
+    return st != LB_OK ? st : waited;
 }
 
 double lb_wetting_h(double theta_deg)
@@ -955,6 +938,37 @@ cudaError_t launch_claim(const DevParams& P, uint8_t* m0, uint8_t* m1, DevPart* 
 }  // namespace lbdp
 
 namespace lbdp {
+
+int queue_fields(lb_handle* h, const double* rho, const double* u, const double* psi, const double* phi)
+{
+    const size_t N = (size_t)h->dp.N;
+    // a non-finite input would spread through the whole box in a few steps:
+    // refuse it before anything is copied
+    const struct {
+        const double* a;
+        size_t n;
+    } in[4] = {{rho, N}, {u, 3 * N}, {psi, N}, {phi, N}};
+    for (const auto& v : in)
+        if (v.a)
+            for (size_t k = 0; k < v.n; ++k)
+                if (!std::isfinite(v.a[k])) return LB_ERR_NONFINITE;
+    cudaSetDevice(h->device);
+    cudaStream_t s = h->stream;
+    double* st_rho = h->staging;
+    double* st_u = h->staging + N;
+    double* st_psi = h->staging + 4 * N;
+    double* st_phi = h->staging + 5 * N;
+    if (rho) LB_TRY(cudaMemcpyAsync(st_rho, rho, N * sizeof(double), cudaMemcpyHostToDevice, s));
+    if (u) LB_TRY(cudaMemcpyAsync(st_u, u, 3 * N * sizeof(double), cudaMemcpyHostToDevice, s));
+    if (psi) LB_TRY(cudaMemcpyAsync(st_psi, psi, N * sizeof(double), cudaMemcpyHostToDevice, s));
+    if (phi) LB_TRY(cudaMemcpyAsync(st_phi, phi, N * sizeof(double), cudaMemcpyHostToDevice, s));
+    // one pass: fields from staging (or current value plus the pending uniform
+    // correction), populations to equilibrium; then the correction is spent
+    LB_TRY(h->ops->set_fields(h->dp, cur_ptrs(h), s, rho ? st_rho : nullptr, u ? st_u : nullptr,
+                              psi ? st_psi : nullptr, phi ? st_phi : nullptr));
+    LB_TRY(cudaMemsetAsync(h->corr, 0, 8 * sizeof(double), s));
+    return LB_OK;
+}
 
 size_t handle_region_bytes(const lb_params* p)
 {

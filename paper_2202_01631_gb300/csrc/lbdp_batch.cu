@@ -733,8 +733,8 @@ int lbs_pump(lbs_server* s, double now, int* active, int* queued)
         it = s->queue.erase(it);
         L.admitted = clock();
         if (st == LB_OK && (!L.q.psi.empty() || !L.q.phi.empty()))
-            st = lb_set_fields(L.h, nullptr, nullptr, L.q.psi.empty() ? nullptr : L.q.psi.data(),
-                               L.q.phi.empty() ? nullptr : L.q.phi.data());
+            st = queue_fields(L.h, nullptr, nullptr, L.q.psi.empty() ? nullptr : L.q.psi.data(),
+                              L.q.phi.empty() ? nullptr : L.q.phi.data());
         for (int k = 0; k < L.q.r.n_particles && st == LB_OK; ++k)
             st = lb_add_particle(L.h, &L.q.r.particles[k], nullptr);
         if (st == LB_OK) st = lbb_set_steps(s->batch, L.h, L.q.r.steps);
