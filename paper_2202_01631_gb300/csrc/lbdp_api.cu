@@ -342,32 +342,34 @@ const SideStream* side_of(const lb_handle* h)
     return h->side.s ? &h->side : (h->batch ? batch_side(h->batch) : nullptr);
 }
 
-// kGraphSteps steps from parity p0 captured on the handle's stream.
-int capture_steps(lb_handle* h, const RowGrid& g, int p0)
+// kGraphSteps steps from parity p0 captured on the handle's stream; false when
+// they cannot be (on the legacy default stream, which a caller can give by its
+// name; without memory for the graph): nothing has run then.
+bool capture_steps(lb_handle* h, const RowGrid& g, int p0)
 {
-    LB_TRY(h->ops->prepare());
     cudaGraph_t graph = nullptr;
-    LB_TRY(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-    int st = LB_OK;
-    for (int t = 0; t < kGraphSteps && st == LB_OK; ++t)
-        st = cuda_status(h->ops->step(h->dp, ptrs(h, (p0 + t) & 1), g, h->stream, side_of(h)));
-    const cudaError_t e = cudaStreamEndCapture(h->stream, &graph);
-    if (st == LB_OK) st = cuda_status(e);
-    if (st == LB_OK) st = cuda_status(cudaGraphInstantiate(&h->gexec[p0], graph, 0));
-    if (graph) cudaGraphDestroy(graph);
-    if (st != LB_OK) {
-        h->gexec[p0] = nullptr;
-        cudaGetLastError();
+    cudaError_t e = h->ops->prepare();
+    if (e == cudaSuccess) e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        for (int t = 0; t < kGraphSteps && e == cudaSuccess; ++t)
+            e = h->ops->step(h->dp, ptrs(h, (p0 + t) & 1), g, h->stream, side_of(h));
+        const cudaError_t end = cudaStreamEndCapture(h->stream, &graph);
+        if (e == cudaSuccess) e = end;
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&h->gexec[p0], graph, 0);
+        if (graph) cudaGraphDestroy(graph);
     }
-    return st;
+    if (e == cudaSuccess) return true;
+    h->gexec[p0] = nullptr;
+    cudaGetLastError();
+    return false;
 }
 
-// Whether lb_step may capture on the handle's stream: not the legacy default
-// stream, and not while the caller is capturing it into a graph of its own
-// (then the plain launches become part of the caller's graph).
+// Whether lb_step may try to capture on the handle's stream: not while the
+// caller is capturing it into a graph of its own (then the plain launches become
+// part of the caller's graph).
 bool can_capture(lb_handle* h)
 {
-    return h->stream && !capturing(h->stream);
+    return !capturing(h->stream);
 }
 
 }  // namespace
@@ -530,13 +532,14 @@ int lb_step(lb_handle* h, int nsteps)
             memcpy(&h->g_dp, &h->dp, sizeof(DevParams));
             h->g_grid = g;
             h->g_steps = 0;
+            h->g_failed = false;
         }
         const bool wait = h->dp.np > 0 && h->g_steps < kGraphAfter && nsteps < kGraphAfter;
         h->g_steps += nsteps;
-        for (; !wait && nsteps - t >= kGraphSteps; t += kGraphSteps) {
-            if (!h->gexec[h->cur]) {
-                const int st = capture_steps(h, g, h->cur);
-                if (st != LB_OK) return st;
+        for (; !wait && !h->g_failed && nsteps - t >= kGraphSteps; t += kGraphSteps) {
+            if (!h->gexec[h->cur] && !capture_steps(h, g, h->cur)) {
+                h->g_failed = true;   // plain launches from here on
+                break;
             }
             LB_TRY(cudaGraphLaunch(h->gexec[h->cur], h->stream));
         }

@@ -160,11 +160,12 @@ struct lb_handle {
     int zplanes[2];   // z chunk length of kz_fused, kz_scalars (0 = size heuristic)
     // lb_step's CUDA graphs of kGraphSteps steps from parity 0 / 1, and the
     // parameters and grids they were captured with (recaptured on a change);
-    // g_steps: steps run with those
+    // g_steps: steps run with those; g_failed: they could not be captured
     cudaGraphExec_t gexec[2];
     lbdp::DevParams g_dp;
     lbdp::RowGrid g_grid;
     long long g_steps;
+    bool g_failed;
     std::vector<lbdp::DevPart> host_parts;
     double rmax;
 };

@@ -1,0 +1,59 @@
+"""Steps where a CUDA graph cannot be captured, and boxes that change after theirs
+was: the bits of plain launches all the same."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2202_01631_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+CUDA_STREAM_LEGACY = 1   # the legacy default stream by its name: it cannot be captured
+PARAMS = dict(W.BASE_PARAMS, nx=24, ny=20, nz=28, periodic=(1, 1, 0), E=0.3, phi_b=1.0, k_d=2e-3)
+SPHERE = dict(pos=(11.3, 9.7, 9.6), R=3.5, m_hat=(0.2, 0.4, -1.0), alpha=1e-2, mu_plus=0.1, mu_minus=-0.1,
+              theta_c_deg=60.0, vel=(0.02, 0.0, 0.01))
+
+
+@pytest.fixture(scope="module")
+def lbdp():
+    from paper_2202_01631_gb300 import build
+    build.build()
+    torch.cuda.init()
+    from paper_2202_01631_gb300 import lbdp as mod
+    return mod
+
+
+def _fill(box, spheres=1):
+    rng = np.random.default_rng(7)
+    shape = box.shape
+    z = np.arange(shape[0])[:, None, None]
+    box.set_fields(rho=1.0 + 0.005 * rng.uniform(-1, 1, shape), u=0.005 * rng.uniform(-1, 1, (3,) + shape),
+                   psi=np.tanh((z - 14.3) / 2.0) + 0.1 * rng.uniform(-1, 1, shape),
+                   phi=1.0 + 0.05 * rng.uniform(-1, 1, shape))
+    for _ in range(spheres):
+        box.add_particle(**SPHERE)
+
+
+def _same(a, b):
+    assert np.array_equal(a.populations(), b.populations()) and np.array_equal(a.mask(), b.mask())
+    fa, fb = a.fields(), b.fields()
+    assert all(np.array_equal(fa[k], fb[k]) for k in fa)
+    for pa, pb in zip(a.particles(), b.particles()):
+        assert all(np.array_equal(pa[k], pb[k]) for k in pa)
+
+
+def _plain(box, steps):
+    for _ in range(steps):
+        box.step(1)   # shorter than a graph
+
+
+@pytest.mark.parametrize("spheres", [0, 1])
+def test_box_on_the_legacy_stream(lbdp, spheres):
+    box = lbdp.Box(precision="fp32", stream=CUDA_STREAM_LEGACY, **PARAMS)
+    ref = lbdp.Box(precision="fp32", **PARAMS)
+    for b in (box, ref):
+        _fill(b, spheres)
+    for n in (200, 60, 5):
+        box.step(n)
+    _plain(ref, 265)
+    _same(box, ref)
