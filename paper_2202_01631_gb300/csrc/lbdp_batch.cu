@@ -164,6 +164,7 @@ struct lbb_batch {
     std::vector<LaunchPlan> plans;
     int par = 0;            // parity of the steps run since the plans were built
     long long ran = 0;      // and their number
+    bool no_graph = false;  // they could not be captured
     int cfg[kNumBatchClasses] = {1, 1};   // z chunks of 16 planes until tuned
     cudaGraphExec_t exec[2] = {nullptr, nullptr};   // graphs starting at parity 0 / 1
     SideStream side{};   // particle kernels, overlapping the fluid kernels
@@ -225,6 +226,7 @@ void rebuild(lbb_batch* b)
     }
     b->par = 0;
     b->ran = 0;
+    b->no_graph = false;
     b->dirty = false;
     drop_graph(b);
 }
@@ -253,30 +255,32 @@ int upload_counts(lbb_batch* b, bool all_one)
     return LB_OK;
 }
 
-int step(lbb_batch* b, int par)
+cudaError_t step(lbb_batch* b, int par)
 {
-    return cuda_status(b->bops->step(b->cfg, b->plans.data(), (int)b->plans.size(), par, b->d_left,
-                                     (int)b->mem.size(), b->stream, &b->side));
+    return b->bops->step(b->cfg, b->plans.data(), (int)b->plans.size(), par, b->d_left, (int)b->mem.size(),
+                         b->stream, &b->side);
 }
 
 // graph_steps steps starting at parity p0 (graph_steps is even, so a launch
-// of it leaves the parity unchanged)
-int capture_graph(lbb_batch* b, int p0)
+// of it leaves the parity unchanged); false when they cannot be captured (on the
+// legacy default stream by its name, without memory for the graph): nothing has
+// run then.
+bool capture_graph(lbb_batch* b, int p0)
 {
-    if (b->exec[p0]) return LB_OK;
+    if (b->exec[p0]) return true;
     cudaGraph_t g = nullptr;
-    LB_TRY(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-    int st = LB_OK;
-    for (int t = 0; t < b->graph_steps && st == LB_OK; ++t) st = step(b, (p0 + t) & 1);
-    cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
-    if (st == LB_OK) st = cuda_status(e2);
-    if (st == LB_OK) st = cuda_status(cudaGraphInstantiate(&b->exec[p0], g, 0));
-    if (g) cudaGraphDestroy(g);
-    if (st != LB_OK) {
-        b->exec[p0] = nullptr;
-        cudaGetLastError();
+    cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        for (int t = 0; t < b->graph_steps && e == cudaSuccess; ++t) e = step(b, (p0 + t) & 1);
+        const cudaError_t end = cudaStreamEndCapture(b->stream, &g);
+        if (e == cudaSuccess) e = end;
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec[p0], g, 0);
+        if (g) cudaGraphDestroy(g);
     }
-    return st;
+    if (e == cudaSuccess) return true;
+    b->exec[p0] = nullptr;
+    cudaGetLastError();
+    return false;
 }
 
 }  // namespace
@@ -470,16 +474,15 @@ int lbb_run(lbb_batch* b, int nsteps, long long* launches)
     if (st != LB_OK) return st;
     // a capture costs about as much as four runs of the graph gain by it: short
     // runs between changes of the batch (requests that come and go) stay plain
-    const bool graph = n >= b->graph_steps && (b->exec[b->par] || n >= 4 * b->graph_steps ||
-                                               b->ran >= 4 * b->graph_steps);
-    const int full = graph ? n / b->graph_steps : 0, rest = n - full * b->graph_steps;
-    if (full > 0) {
-        st = capture_graph(b, b->par);
-        if (st != LB_OK) return st;
-        for (int k = 0; k < full; ++k) LB_TRY(cudaGraphLaunch(b->exec[b->par], b->stream));
+    bool graph = !b->no_graph && n >= b->graph_steps &&
+                 (b->exec[b->par] || n >= 4 * b->graph_steps || b->ran >= 4 * b->graph_steps);
+    if (graph && !capture_graph(b, b->par)) {
+        b->no_graph = true;   // plain launches until the batch changes
+        graph = false;
     }
-    for (int k = 0; k < rest && st == LB_OK; ++k) st = step(b, (b->par + k) & 1);
-    if (st != LB_OK) return st;
+    const int full = graph ? n / b->graph_steps : 0, rest = n - full * b->graph_steps;
+    for (int k = 0; k < full; ++k) LB_TRY(cudaGraphLaunch(b->exec[b->par], b->stream));
+    for (int k = 0; k < rest; ++k) LB_TRY(step(b, (b->par + k) & 1));
     b->par = (b->par + n) & 1;
     b->ran += n;
     for (Member& m : b->mem) {

@@ -57,3 +57,22 @@ def test_box_on_the_legacy_stream(lbdp, spheres):
         box.step(n)
     _plain(ref, 265)
     _same(box, ref)
+
+
+@pytest.mark.parametrize("calls", [(40,), (5, 12, 9, 8, 6)])
+def test_batch_on_the_legacy_stream(lbdp, calls):
+    batch = lbdp.Batch(precision="fp32", arena_bytes=1 << 28, graph_steps=4, stream=CUDA_STREAM_LEGACY)
+    try:
+        boxes = [batch.add_box(**PARAMS) for _ in range(2)]
+        for k, b in enumerate(boxes):
+            _fill(b, k)
+            batch.set_steps(b, 40 - 9 * k)
+        for n in calls:
+            batch.run(n)
+        for k, b in enumerate(boxes):
+            ref = lbdp.Box(precision="fp32", **PARAMS)
+            _fill(ref, k)
+            _plain(ref, 40 - 9 * k)
+            _same(b, ref)
+    finally:
+        batch.close()
