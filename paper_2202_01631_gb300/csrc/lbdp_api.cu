@@ -327,15 +327,6 @@ bool graph_pays(const DevParams& P, bool fp64) { return P.np == 0 || P.N <= (fp6
 
 bool same_grid(const dim3& a, const dim3& b) { return a.x == b.x && a.y == b.y && a.z == b.z; }
 
-// Whether a capture is under way on s (calls that set a box up refuse then).
-bool capturing(cudaStream_t s)
-{
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
-    cudaGetLastError();
-    return true;
-}
-
 // Streams beside the box's own for the particle kernels of its steps.
 const SideStream* side_of(const lb_handle* h)
 {
@@ -941,6 +932,14 @@ cudaError_t launch_claim(const DevParams& P, uint8_t* m0, uint8_t* m1, DevPart* 
 }  // namespace lbdp
 
 namespace lbdp {
+
+bool capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
 
 int queue_fields(lb_handle* h, const double* rho, const double* u, const double* psi, const double* phi)
 {

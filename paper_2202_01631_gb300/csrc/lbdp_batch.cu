@@ -470,6 +470,10 @@ int lbb_run(lbb_batch* b, int nsteps, long long* launches)
     const int n = (int)std::min<long long>(nsteps, most);
     if (n == 0) return LB_OK;
     if (plans_stale(b)) rebuild(b);
+    // the caller is capturing the stream: a run of whole graphs not yet captured
+    // cannot be recorded (its step counts come from memory that does not outlive
+    // the call)
+    if (n >= b->graph_steps && !b->exec[b->par] && capturing(b->stream)) return LB_ERR_CUDA;
     int st = upload_counts(b, false);
     if (st != LB_OK) return st;
     // a capture costs about as much as four runs of the graph gain by it: short

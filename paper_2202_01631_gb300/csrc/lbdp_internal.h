@@ -111,6 +111,8 @@ cudaError_t launch_claim(const DevParams& P, uint8_t* m0, uint8_t* m1, DevPart* 
 size_t handle_region_bytes(const lb_params* p);
 DevPtrs handle_ptrs(const lb_handle* h, int src);
 int lb_create_in(const lb_params* p, lbb_batch* batch, void* region, lb_handle** out);
+// Whether a capture is under way on s (calls that set a box up refuse then).
+bool capturing(cudaStream_t s);
 // lb_set_fields without its wait: the arrays must live until the stream has
 // copied them.
 int queue_fields(lb_handle* h, const double* rho, const double* u, const double* psi, const double* phi);

@@ -76,3 +76,26 @@ def test_batch_on_the_legacy_stream(lbdp, calls):
             _same(b, ref)
     finally:
         batch.close()
+
+
+def test_batch_refuses_whole_graphs_under_capture(lbdp):
+    stream = torch.cuda.Stream()
+    batch = lbdp.Batch(precision="fp32", arena_bytes=1 << 28, graph_steps=4, stream=stream.cuda_stream)
+    try:
+        box = batch.add_box(**PARAMS)
+        _fill(box)
+        batch.set_steps(box, 50)
+        stream.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+            for n in (4, 15, 50):
+                with pytest.raises(lbdp.LbError):
+                    batch.run(n)
+        assert batch.steps_left(box) == 50
+        batch.run(50)
+        ref = lbdp.Box(precision="fp32", **PARAMS)
+        _fill(ref)
+        _plain(ref, 50)
+        _same(box, ref)
+    finally:
+        batch.close()
