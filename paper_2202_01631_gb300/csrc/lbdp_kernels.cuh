@@ -242,13 +242,32 @@ __device__ __forceinline__ int dir_comp(int i)
     return (int)((t >> (2 * i)) & 3ull) - 1;
 }
 
-// 1 / sqrt(a): the CUDA function in FP64; in FP32 the CUDA function and one
-// Newton-Raphson step y (3 - a y^2) / 2, within an ulp.
-__device__ __forceinline__ double inv_sqrt(double a) { return rsqrt(a); }
-__device__ __forceinline__ float inv_sqrt(float a)
+// d / sqrt(a) rounded once (within 0.5001 ulp), for components of a unit vector:
+// y is CUDA's FP32 inverse square root, e = 1 - a y^2 its residual, taken with
+// the rounding of a y as a second term, and 1 / sqrt(a) = y (1 - e)^(-1/2) =
+// y (1 + c) by the binomial series (|e| < 2^-20: two terms in FP64, one in FP32);
+// the quotient adds d y's rounding and c d y to d y.  An IEEE square root and a
+// division round twice and take longer: measured on GB300, a step with one
+// sphere, FP32 24^3 46.7 us (IEEE 49.8), 128^3 188.5 (196.9); FP64 32^3 175.9
+// (180.3), 96^3 1448 (1469).  Errors over random link points, largest and mean,
+// in units of the rounding: ghost FP32 4.69, 0.393 (IEEE 5.38, 0.445), FP64 4.54,
+// 0.391 (4.89, 0.437); slip FP32 8.14, 0.461 (10.16, 0.519), FP64 6.10, 0.458
+// (7.85, 0.511).
+template <class R>
+struct InvNorm {
+    R y, c;
+    __device__ __forceinline__ R times(R d) const
+    {
+        const R q = mul_x(d, y);
+        return add_x(q, fma_x(c, q, fma_x(d, y, -q)));
+    }
+};
+template <class R>
+__device__ __forceinline__ InvNorm<R> inv_norm(R a)
 {
-    const float y = rsqrtf(a);
-    return mul_x(y, fma_x(mul_x(-0.5f * a, y), y, 1.5f));
+    const R y = (R)rsqrtf((float)a), t = mul_x(a, y), tl = fma_x(a, y, -t);
+    const R e = fma_x(-tl, y, fma_x(-t, y, (R)1));
+    return {y, sizeof(R) == 4 ? mul_x((R)0.5, e) : mul_x(e, fma_x((R)0.375, e, (R)0.5))};
 }
 
 // The wetting ghosts of fluid node (x, y, z) on its links into particle q (bit
@@ -257,8 +276,7 @@ __device__ __forceinline__ float inv_sqrt(float a)
 // at a sphere's surface hold different links, and a body per direction, taken
 // by whichever lane needs it, made the blocks of kz_fused next to a sphere
 // run twice as long as the rest of the grid (latency of its square root,
-// division and particle loads, 18 times per slot).  In FP32 two links go
-// through each iteration, for the latency of the inverse square root.
+// division and particle loads, 18 times per slot).
 // Measured on GB300, FP32, loop against unrolled bodies: kz_fused 201 -> 131
 // us with one sphere R = 8 in 128^3, 66 -> 42 us in 24^3.
 template <class R, class Q>
@@ -271,27 +289,21 @@ __device__ __forceinline__ void psi_ghosts(const DevParams& P, const Q& q, int x
     int_offset(P, q.g, x, y, z, D);
     R r0[3];   // x - X
     link_offset_r<R>(q.g, D, 0, r0);
-    constexpr int U = sizeof(R) == 4 ? 2 : 1;
-    while (bits) {
-#pragma unroll
-        for (int k = 0; k < U; ++k) {
-            // no link left: direction 0, whose ghost c . n_hat is 0
-            const int i = bits ? __ffs((int)bits) - 1 : 0;
-            bits &= bits - 1;
-            const R c0 = (R)dir_comp<0>(i), c1 = (R)dir_comp<1>(i), c2 = (R)dir_comp<2>(i);
-            const R r[3] = {fma_x((R)0.5, c0, r0[0]), fma_x((R)0.5, c1, r0[1]), fma_x((R)0.5, c2, r0[2])};
-            const R gd = mul_x(mul_x(Hk, dot_x(c0, c1, c2, r[0], r[1], r[2])),
-                               inv_sqrt(dot_x(r[0], r[1], r[2], r[0], r[1], r[2])));
-            const R ax = i < 7 ? gd : (R)0, dg = i < 7 ? (R)0 : gd;
-            s.sa += ax;
-            s.sd += dg;
-            s.ga[0] = fma_x(c0, ax, s.ga[0]);
-            s.ga[1] = fma_x(c1, ax, s.ga[1]);
-            s.ga[2] = fma_x(c2, ax, s.ga[2]);
-            s.gd[0] = fma_x(c0, dg, s.gd[0]);
-            s.gd[1] = fma_x(c1, dg, s.gd[1]);
-            s.gd[2] = fma_x(c2, dg, s.gd[2]);
-        }
+    for (; bits; bits &= bits - 1) {
+        const int i = __ffs((int)bits) - 1;
+        const R c0 = (R)dir_comp<0>(i), c1 = (R)dir_comp<1>(i), c2 = (R)dir_comp<2>(i);
+        const R r[3] = {fma_x((R)0.5, c0, r0[0]), fma_x((R)0.5, c1, r0[1]), fma_x((R)0.5, c2, r0[2])};
+        const R gd = mul_x(Hk, inv_norm(dot_x(r[0], r[1], r[2], r[0], r[1], r[2]))
+                                   .times(dot_x(c0, c1, c2, r[0], r[1], r[2])));
+        const R ax = i < 7 ? gd : (R)0, dg = i < 7 ? (R)0 : gd;
+        s.sa += ax;
+        s.sd += dg;
+        s.ga[0] = fma_x(c0, ax, s.ga[0]);
+        s.ga[1] = fma_x(c1, ax, s.ga[1]);
+        s.ga[2] = fma_x(c2, ax, s.ga[2]);
+        s.gd[0] = fma_x(c0, dg, s.gd[0]);
+        s.gd[1] = fma_x(c1, dg, s.gd[1]);
+        s.gd[2] = fma_x(c2, dg, s.gd[2]);
     }
 }
 

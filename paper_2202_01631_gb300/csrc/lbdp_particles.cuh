@@ -207,10 +207,11 @@ __device__ __forceinline__ R link_slip(const NodeLinks<R>& l, int i, const R gph
     const R mp = PartR<R>::mu_p(l.q), mm = PartR<R>::mu_m(l.q);
     if (mp == (R)0 && mm == (R)0) return (R)0;
     const R mu = mp == mm ? mp : (cap_minus_at(l.q, l.D, k0, k1, k2) ? mm : mp);
-    const R is = inv_sqrt(dot_x(r[0], r[1], r[2], r[0], r[1], r[2]));
-    const R cn = mul_x(dot_x(c0, c1, c2, r[0], r[1], r[2]), is);
-    const R gn = mul_x(dot_x(gphi[0], gphi[1], gphi[2], r[0], r[1], r[2]), is);
-    return mul_x(mu, fma_x(-cn, gn, dot_x(c0, c1, c2, gphi[0], gphi[1], gphi[2])));
+    const InvNorm<R> in = inv_norm(dot_x(r[0], r[1], r[2], r[0], r[1], r[2]));
+    const R n0 = in.times(r[0]), n1 = in.times(r[1]), n2 = in.times(r[2]);
+    const R ng = dot_x(n0, n1, n2, gphi[0], gphi[1], gphi[2]);
+    return dot_x(c0, c1, c2, mul_x(mu, fma_x(-n0, ng, gphi[0])), mul_x(mu, fma_x(-n1, ng, gphi[1])),
+                 mul_x(mu, fma_x(-n2, ng, gphi[2])));
 }
 
 // c . u_b of link i, u_b = U + Omega x r + v_s.
