@@ -694,13 +694,13 @@ __device__ __forceinline__ double rotate_unit(const double (&m)[3], const double
     const double w2 = dot_x(w[0], w[1], w[2], w[0], w[1], w[2]);
     double s1, c1, cw;
     if (w2 < 0.01) {
-        // products with the rounded reciprocals: the divisions would be ten
-        // dependent chains on the FP64 pipe.  Lane 0: s1, others: 2 c1
-        const bool s = lane == 0;
-        const double k0 = s ? 1.0 / 6.0 : 1.0 / 12.0, k1 = s ? 1.0 / 20.0 : 1.0 / 30.0, k2 = s ? 1.0 / 42.0 : 1.0 / 56.0,
-                     k3 = s ? 1.0 / 72.0 : 1.0 / 90.0, k4 = s ? 1.0 / 110.0 : 1.0 / 132.0;
-        const double t =
-            fma_x(-w2 * k0, fma_x(-w2 * k1, fma_x(-w2 * k2, fma_x(-w2 * k3, fma_x(-w2 * k4, 1.0, 1.0), 1.0), 1.0), 1.0), 1.0);
+        // s1 = 1 - w2/6 (1 - w2/20 (...)) in the even lanes, 2 c1 = 1 - w2/12 (1 -
+        // w2/30 (...)) in the odd ones.  The ten quotients w2 / (k + 2)(k + 3) are
+        // a lane's each: one division instead of a chain of five
+        const double d = -w2 / (double)((lane + 2) * (lane + 3));
+        double t = 1.0;
+#pragma unroll
+        for (int k = 4; k >= 0; --k) t = fma_x(__shfl_sync(0xffffffffu, d, 2 * k + (lane & 1)), t, 1.0);
         s1 = __shfl_sync(0xffffffffu, t, 0);
         c1 = 0.5 * __shfl_sync(0xffffffffu, t, 1);
         cw = fma_x(-w2, c1, 1.0);
