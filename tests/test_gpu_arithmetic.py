@@ -22,6 +22,22 @@ static __global__ void k_over(const R* a, const R* d, R* q, int n)
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
         q[i] = inv_norm(a[i]).times(d[i]);
 }
+// every value of binade ex, both signs: how many differ from the rounded quotient
+static __global__ void k_recip(int ex, unsigned long long* bad)
+{
+    for (unsigned m = blockIdx.x * blockDim.x + threadIdx.x; m < (1u << 23); m += gridDim.x * blockDim.x) {
+        const float a = __uint_as_float((unsigned)(ex + 127) << 23 | m);
+        const Vec<float, 2> r = recip(Vec<float, 2>{make_float2(a, -a)});
+        if (__float_as_uint(r.v.x) != __float_as_uint(__frcp_rn(a)) ||
+            __float_as_uint(r.v.y) != __float_as_uint(__frcp_rn(-a)))
+            atomicAdd(bad, 1ull);
+    }
+}
+extern "C" int recip32(int ex, unsigned long long* bad)
+{
+    k_recip<<<1024, 256>>>(ex, bad);
+    return (int)cudaDeviceSynchronize();
+}
 extern "C" int over32(const float* a, const float* d, float* q, int n)
 {
     k_over<float><<<1024, 256>>>(a, d, q, n);
@@ -76,3 +92,12 @@ def test_quotient_by_a_norm(lib, bits, slack):
     r = np.where(r.astype(wide) > np.abs(x), np.nextafter(r, dtype(0)), r)
     err = np.abs(got.astype(wide) - x) / np.spacing(r).astype(wide)
     assert float(err[4:].max()) <= 0.5 + slack
+
+
+def test_reciprocal_of_a_density_is_the_rounded_quotient(lib):
+    bad = torch.zeros(1, dtype=torch.int64, device="cuda")
+    torch.cuda.synchronize()
+    lib.recip32.argtypes = [C.c_int, C.c_void_p]
+    for ex in range(-126, 126):
+        assert lib.recip32(ex, bad.data_ptr()) == 0
+        assert int(bad.item()) == 0, ex
