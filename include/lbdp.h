@@ -189,9 +189,9 @@ int lb_profile_step(lb_handle* h, int nsteps, double* ms, int* launches);
  * force and collide-stream, and the psi/phi transport) march along z through
  * 32 x 8 column tiles; a block takes one z chunk.  Short chunks recompute
  * more halo planes, long ones leave SMs idle, and the best length depends on
- * the box, so lb_tune times each kernel alone over reps launches for chunk
- * lengths from 4 to 64 planes (each rounded to equal chunks) and keeps the
- * fastest per kernel.  The kernels only rewrite the next step's buffers and
+ * the box, so lb_tune times each kernel alone over reps launches for the
+ * lengths the library chooses by size and others from 1 to 64 planes (each
+ * rounded to equal chunks) and keeps the fastest per kernel.  The kernels only rewrite the next step's buffers and
  * the stored velocity, which is saved and restored: the state is unchanged,
  * and the results of later steps do not depend on the chunk length (bit for
  * bit).  planes_out[2], ms_out[2] (optional): the chosen lengths and their

@@ -581,11 +581,13 @@ int lb_tune(lb_handle* h, int reps, int planes_out[2], double ms_out[2])
     // kz_fused rewrites the stored velocity of the bulk nodes: keep a copy
     const size_t ub = 3 * (size_t)P.N * h->ops->fld_bytes;
     LB_TRY(cudaMemcpyAsync(h->staging, h->u, ub, cudaMemcpyDeviceToDevice, s));
-    // candidate chunk lengths, each kept once after rounding to equal chunks
-    static const int kCand[] = {4, 6, 8, 12, 16, 24, 32, 48, 64};
+    // candidate chunk lengths, each kept once after rounding to equal chunks: the
+    // library's own choices, and one plane to 64
+    const bool fp64 = h->prm.precision == LB_FP64;
+    const int lengths[] = {default_fused_planes(P, fp64 ? 1 : 2), default_scalar_planes(P, fp64),
+                           1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64};
     std::vector<int> cand;
-    for (int c : kCand) {
-        if (c > P.nz && !cand.empty()) break;
+    for (int c : lengths) {
         const int p = (int)zm_grid(P, c).z;
         const int planes = (P.nz + p - 1) / p;
         if (std::find(cand.begin(), cand.end(), planes) == cand.end()) cand.push_back(planes);
