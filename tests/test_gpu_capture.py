@@ -99,3 +99,30 @@ def test_batch_refuses_whole_graphs_under_capture(lbdp):
         _same(box, ref)
     finally:
         batch.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_box_changed_after_its_graph_was_captured(lbdp, precision):
+    """Chunk lengths on either side of the 152 blocks up to which covering starts
+    early (2 x 3 x 28 and 2 x 3 x 14), a second, larger sphere, a checkpoint."""
+    params = dict(PARAMS, nx=40, nz=28, ny=20)
+    boxes = [lbdp.Box(precision=precision, **params) for _ in range(2)]
+    for b in boxes:
+        _fill(b)
+    captured, plain = boxes
+
+    def both(what):
+        for b in boxes:
+            what(b)
+        captured.step(131)   # whole graphs and a few plain steps, the parity changing
+        _plain(plain, 131)
+        _same(captured, plain)
+
+    both(lambda b: None)
+    both(lambda b: b.set_planes(0, 1))
+    both(lambda b: b.set_planes(1, 2))
+    both(lambda b: b.add_particle(pos=(29.6, 10.4, 16.2), R=4.6, m_hat=(1.0, 0.1, 0.3), alpha=1e-2, omega=(0.0, 0.01, 0.0)))
+    blobs = [b.save_state() for b in boxes]
+    both(lambda b: b.set_planes(0, 0))
+    both(lambda b: b.load_state(blobs[boxes.index(b)]))
+    assert len(captured.particles()) == 2
