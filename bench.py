@@ -72,7 +72,7 @@ def parse():
     ap.add_argument("--scalar-scheme", type=int, default=0, choices=[0, 1],
                     help="psi/phi transport: 0 finite differences, 1 D3Q7 lattice Boltzmann")
     ap.add_argument("--no-cpu-baseline", action="store_true")
-    ap.add_argument("--no-tune", action="store_true", help="single form: keep the size heuristic's z chunks")
+    ap.add_argument("--no-tune", action="store_true", help="single form: keep the z chunks chosen by size")
     ap.add_argument("--form", default="single", choices=["single", "batched", "served"])
     ap.add_argument("--boxes", type=int, default=64, help="batched form: number of boxes")
     ap.add_argument("--graph-steps", type=int, default=16,

@@ -160,13 +160,14 @@ int lb_add_particle(lb_handle* h, const lb_particle_desc* desc, int* id_out);
  * without waiting.  Each step: chemical potentials (Eq. chem_potentials);
  * force, streaming with bounce-back and BGK collision; psi/phi transport
  * (Eq. diffusion_reaction); particle update; covering/uncovering.  The
- * particle kernels run on a second stream of the library's that joins the
+ * particle kernels run on two more streams of the library's that join the
  * handle's stream before each step ends.  Whole groups of 8 steps run as one
  * captured CUDA graph for a box without particles, and for a small one with
- * particles once it has run 128 steps (captured on first use and again after
- * the parameters or launch grids change); while the caller is
- * itself capturing the handle's stream, and on the legacy default stream,
- * every step is launched plainly.  Results do not depend on the route. */
+ * particles once it has run 128 steps in calls of 8 or more, or when one call
+ * asks for 128 (captured on first use and again after the parameters or launch
+ * grids change); while the caller is itself capturing the handle's stream, and
+ * where a capture fails (on the legacy default stream), every step is launched
+ * plainly.  Results do not depend on the route. */
 int lb_step(lb_handle* h, int nsteps);
 
 /* Run nsteps steps like lb_step, but with every kernel on the handle's stream

@@ -47,7 +47,7 @@ int reduction_blocks(const lb_params* p)
 {
     long long N = (long long)p->nx * p->ny * p->nz;
     long long b = (N + 255) / 256;
-    return (int)(b < 152 * 8 ? b : 152 * 8);
+    return (int)(b < kSMs * 8 ? b : kSMs * 8);
 }
 
 // Every array of a box in one region, each start aligned to 256 bytes.  With
@@ -170,10 +170,11 @@ int default_fused_planes(const DevParams& P, int halves)
         const long long blocks = cols * chunks;
         double cost;
         if (halves == 2) {
-            const double waves = blocks <= 152 ? 0.7 : blocks <= 304 ? 1.0 : blocks <= 608 ? 2.0 : (double)blocks / 304;
+            const double waves = blocks <= kSMs ? 0.7 : blocks <= 2 * kSMs ? 1.0 : blocks <= 4 * kSMs ? 2.0
+                                                                                      : (double)blocks / (2 * kSMs);
             cost = (waves + (P.np > 0 ? 1.5 : 0.5)) * ((p + 1) / 2 + 3);
         } else {
-            const long long n = (blocks + 151) / 152;
+            const long long n = (blocks + kSMs - 1) / kSMs;
             cost = (n % 2 ? (double)n + 0.3 : (double)n) * (p + 1.3);
         }
         if (cost < best) {
@@ -200,8 +201,8 @@ int default_scalar_planes(const DevParams& P, bool fp64)
         const int chunks = (P.nz + p - 1) / p;
         if ((P.nz + chunks - 1) / chunks != p) continue;   // not the length of equal chunks
         const long long blocks = cols * chunks;
-        const double cost = fp64 ? ((double)((blocks + 151) / 152) + 0.3) * (p + 1.3)
-                                 : (std::max(0.5, (double)blocks / 456) + 1.0) * (p + 5);
+        const double cost = fp64 ? ((double)((blocks + kSMs - 1) / kSMs) + 0.3) * (p + 1.3)
+                                 : (std::max(0.5, (double)blocks / (3 * kSMs)) + 1.0) * (p + 5);
         if (cost < best) {
             best = cost;
             planes = p;
@@ -311,9 +312,9 @@ int read_err(lb_handle* h)
 
 
 // Steps per captured graph of lb_step (even: a launch leaves the parity), and
-// the steps a box with particles runs plainly before its graph is captured: the
-// capture of eight steps of nine kernels costs about as much as a hundred steps
-// gain by it.
+// the steps (in calls of kGraphSteps or more) a box with particles runs plainly
+// before its graph is captured, unless one call asks for as many: the capture of
+// eight steps of nine kernels costs about as much as a hundred steps gain by it.
 constexpr int kGraphSteps = 8, kGraphAfter = 128;
 
 // Whether graph launches beat plain ones.  Without particles they do (measured
@@ -918,7 +919,7 @@ namespace lbdp {
 cudaError_t launch_bflag(const DevParams& P, const uint8_t* mask, uint8_t* bflag, cudaStream_t s)
 {
     long long b = (P.N + 255) / 256;
-    int blocks = (int)(b < 152 * 16 ? b : 152 * 16);
+    int blocks = (int)(b < kSMs * 16 ? b : kSMs * 16);
     k_bflag_all<<<blocks, 256, 0, s>>>(P, mask, bflag);
     return cudaGetLastError();
 }
@@ -927,7 +928,7 @@ cudaError_t launch_claim(const DevParams& P, uint8_t* m0, uint8_t* m1, DevPart* 
                          long long* nfluid, cudaStream_t s)
 {
     long long b = (P.N + 255) / 256;
-    int blocks = (int)(b < 152 * 16 ? b : 152 * 16);
+    int blocks = (int)(b < kSMs * 16 ? b : kSMs * 16);
     k_claim<<<blocks, 256, 0, s>>>(P, m0, m1, parts, p, q, nfluid);
     return cudaGetLastError();
 }
@@ -1085,7 +1086,7 @@ int lb_create_in(const lb_params* p, lbb_batch* batch, void* region, lb_handle**
     if (e == cudaSuccess) {
         // populations from rho = rho0 everywhere (staging holds rho0)
         const long long b = (P.N + 255) / 256;
-        k_rest<<<(int)(b < 152 * 16 ? b : 152 * 16), 256, 0, s>>>(h->staging, p->rho0, P.N, h->nfluid);
+        k_rest<<<(int)(b < kSMs * 16 ? b : kSMs * 16), 256, 0, s>>>(h->staging, p->rho0, P.N, h->nfluid);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = h->ops->set_fields(P, cur_ptrs(h), s, h->staging, nullptr, nullptr, nullptr);
         if (e == cudaSuccess && !batch) e = cudaStreamSynchronize(s);

@@ -51,7 +51,7 @@ struct PrecOps {
     // one full time step (fluid kernels, then particle kernels when np > 0)
     cudaError_t (*step)(const DevParams&, const DevPtrs&, const RowGrid&, cudaStream_t, const SideStream*);
     // the same step with an event recorded before the first kernel and after
-    // each kernel class: ev[0..5] around mu, links, collide, scalars, cover
+    // each kernel class: ev[0..5] around the classes of KernelClass
     cudaError_t (*step_events)(const DevParams&, const DevPtrs&, const RowGrid&, cudaStream_t, cudaEvent_t* ev);
     // one bulk kernel alone over grid: which 0 kz_fused, 1 kz_scalars
     cudaError_t (*bulk)(int which, const DevParams&, const DevPtrs&, dim3 grid, cudaStream_t);
@@ -159,7 +159,7 @@ struct lb_handle {
     double* red_part;
     double* red_out;
     int red_blocks;
-    int zplanes[2];   // z chunk length of kz_fused, kz_scalars (0 = size heuristic)
+    int zplanes[2];   // z chunk length of kz_fused, kz_scalars (0 = chosen by size)
     // lb_step's CUDA graphs of kGraphSteps steps from parity 0 / 1, and the
     // parameters and grids they were captured with (recaptured on a change);
     // g_steps: steps run with those; g_failed: they could not be captured

@@ -463,14 +463,9 @@ __device__ void block_sum(double (&v)[K], double* smem /* [32*K] */)
 // their K values as rows, in thread order, into shared memory; G threads per
 // value add rows g, g + G, ..., and thread k adds its G partials in order.
 // The order depends only on which threads contribute, so the result is
-// deterministic.  It is valid in thread 0's v and stays in sm[0..K-1]; sm
-// holds block_rows_bytes<K>(blockDim.x) bytes (results, 32 warp counts and
-// the G x K partials below sm[256], rows from there).  blockDim.x >= G K.
-template <int K>
-__host__ __device__ constexpr int block_rows_groups()
-{
-    return K > 16 ? 4 : 16;
-}
+// deterministic.  It is left in sm[0..K-1]; sm holds
+// block_rows_bytes<K>(blockDim.x) bytes (results, 32 warp counts and the G x K
+// partials below sm[256], rows from there).  blockDim.x >= G K.
 template <int K>
 __host__ __device__ constexpr size_t block_rows_bytes(int threads)
 {
@@ -478,10 +473,10 @@ __host__ __device__ constexpr size_t block_rows_bytes(int threads)
 }
 
 template <int K>
-__device__ void block_sum_rows(double (&v)[K], double* sm)
+__device__ void block_sum_rows(const double (&v)[K], double* sm)
 {
-    constexpr int G = block_rows_groups<K>();
-    static_assert(K <= 64 && G * K <= 176, "reduction layout");
+    constexpr int G = 16;
+    static_assert(G * K <= 176, "reduction layout");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     int* wcount = (int*)(sm + 64);
     double* part = sm + 80;
@@ -518,10 +513,6 @@ __device__ void block_sum_rows(double (&v)[K], double* sm)
         for (int g = 0; g < G; ++g) s += part[g * K + t];
         sm[t] = s;
     }
-    __syncthreads();
-    if (t == 0)
-#pragma unroll
-        for (int k = 0; k < K; ++k) v[k] = sm[k];
     __syncthreads();
 }
 

@@ -25,6 +25,8 @@ constexpr int kMaxParticles = 64;
 // is kept as its four independent numbers (p_iso, grad psi).
 constexpr int kPtFields = 4;
 
+constexpr int kSMs = 152;   // of a GB300
+
 // Arithmetic with its rounding written out.  The particle sums and solve,
 // the boundary velocities and the refill of uncovered nodes are inlined into
 // the single-box and the batched kernels; with every multiply-add fused or

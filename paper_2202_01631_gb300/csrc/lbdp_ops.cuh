@@ -52,9 +52,9 @@ inline void side_launch_early(void (*k)(A...), dim3 grid, int threads, const Sid
     side_launch_with(at, 2, side->s, k, grid, threads, side, args...);
 }
 
-// Blocks of kz_scalars (at most one on each of the 152 SMs) up to which
-// k_cover_apply is launched early.
-constexpr unsigned kEarlyCoverBlocks = 152;
+// Blocks of kz_scalars (at most one on each SM) up to which k_cover_apply is
+// launched early.
+constexpr unsigned kEarlyCoverBlocks = kSMs;
 
 template <class C>
 struct Ops {
@@ -185,7 +185,7 @@ struct Ops {
     static int grid1d(const DevParams& P)
     {
         long long b = (P.N + 255) / 256;
-        return (int)(b < 152 * 16 ? b : 152 * 16);
+        return (int)(b < kSMs * 16 ? b : kSMs * 16);
     }
 
     static cudaError_t set_fields(const DevParams& P, const DevPtrs& D, cudaStream_t s, const double* rho,
@@ -339,7 +339,6 @@ struct BOps {
         BatchOps t;
         t.prepare = &prepare;
         t.node = &node;
-        t.prepare = &prepare;
         t.step = &step;
         return t;
     }

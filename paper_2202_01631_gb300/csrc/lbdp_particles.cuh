@@ -137,7 +137,7 @@ __device__ __forceinline__ unsigned links_into(const Around& a, int k)
     return b;
 }
 
-// grad phi of the node (as grad_phi_at) from differences to its own value;
+// grad phi of the node, 3 sum_i w_i c_i phi(x + c_i), from differences to its own value;
 // stopped directions carry the node's own value.
 template <class R, class F>
 __device__ __forceinline__ void grad_phi_around(const Around& a, const F* phi, int n, R own, R dphi, R g[3])
@@ -177,8 +177,7 @@ __device__ __forceinline__ void node_links(const DevParams& P, const DevPart& pa
     link_offset_r<R>(l.q.g, l.D, 0, l.r0);
 }
 
-// m . r <= 0 at the midpoint of link (c0, c1, c2), the oracle's decision (as
-// cap_minus, for a direction known at run time).
+// m . r <= 0 at the midpoint of link (c0, c1, c2), the oracle's decision.
 template <class Q>
 __device__ __forceinline__ bool cap_minus_at(const Q& q, const int D[3], int c0, int c1, int c2)
 {
@@ -319,8 +318,8 @@ __device__ __forceinline__ void link_box(const DevPart& q, int o[3])
     for (int a = 0; a < 3; ++a) o[a] = q.g.Xi[a] - q.Rc - 2;
 }
 
-// F at the fluid nodes next to particle p (those whose lowest adjacent
-// particle is p, as in k_collide_particles), into the force array.
+// F at the fluid nodes of particle p's link box that lie next to a particle, into
+// the force array.
 template <class C>
 __device__ __forceinline__ void f_part_block(const DevParams& P, const DevPtrs& D, int p, int bi, int nbi,
                                              NodeList<C>& list)
@@ -336,8 +335,8 @@ __device__ __forceinline__ void f_part_block(const DevParams& P, const DevPtrs& 
             const int n = list.n[e];
             int x, y, z;
             node_coords(P, n, x, y, z);
-            // a node next to several particles: each of their blocks writes the
-            // same force
+            // a node in the boxes of several particles: each of their blocks
+            // writes the same force
             const size_t N = (size_t)P.N;
             const F* pt = (const F*)D.pt;
             GAcc<F, kPtFields> a;

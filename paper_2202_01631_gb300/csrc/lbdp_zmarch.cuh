@@ -619,7 +619,7 @@ __device__ __forceinline__ void force_plane(const R* pa, const R* pb, int s1, R 
     }
 }
 
-// BGK collision with Guo forcing of NP nodes, as collide_store, with the
+// BGK collision with Guo forcing of NP nodes, with the
 // populations of a weight class scaled by its weight: for c of diagonal
 // weight w, g* = (1 - 1/tau) g + (T_c + e) +- h.c with
 //   T_c = cu (c.v), v = w (4.5 rho u / tau + 9 (1 - 1/(2 tau)) F),

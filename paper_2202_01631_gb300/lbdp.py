@@ -249,7 +249,7 @@ def lb_tune(h, reps: int = 10):
 
 
 def lb_set_planes(h, fused: int, scalars: int) -> None:
-    """Chunk lengths of the two bulk kernels (0 = size heuristic)."""
+    """Chunk lengths of the two bulk kernels (0 = chosen by size)."""
     planes = (C.c_int * 2)(int(fused), int(scalars))
     _check(_lib.lb_set_planes(h, planes), "lb_set_planes")
 
