@@ -303,10 +303,12 @@ def traffic_record(kernel, precision, workload_name):
 
 
 def source_hash():
+    """Of the files the single-box kernels are compiled from: host code (the C
+    API, batches and their interface) does not void a capture."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2202_01631_gb300", "csrc")
     for name in sorted(os.listdir(csrc)):
-        if name.endswith((".cu", ".cuh", ".h")):
+        if name.endswith(".cuh") or name.startswith("lbdp_prec_"):
             with open(os.path.join(csrc, name), "rb") as f:
                 h.update(name.encode() + f.read())
     return h.hexdigest()[:16]
