@@ -153,12 +153,13 @@ DevPtrs cur_ptrs(const lb_handle* h)
 // barriers and takes 1.3 of its share), plus 1.3 per block for the recomputed
 // halo planes; within 5% of the best length over ten boxes of 32^3 to 133^3
 // (without the odd block's price 16%).
-// Measured on GB300 over 1 to 128 planes (us, choice in brackets): FP32 with a
-// sphere 24^3 2 planes 31, 6 planes 44 [1]; 128^3 4 planes 123, 6 110, 8 115,
-// 12 128 [8]; 256^3 8 planes 668, 24 603, 32 597, 64 623 [32]; without one 64^3
-// 2 planes 26, 4 20, 16 31 [4]; 80 x 76 x 84 4 planes 51, 10 42, 24 57 [10];
-// FP64 32^3 1 plane 115, 6 planes 333 [1]; 96^3 4 planes 945, 8 875, 12 861, 16
-// 1118 [12]; 102 x 107 x 95 12 planes 1439, 16 1616, 19 1383 [19].
+// Measured on GB300 (us per launch by planes, the choice in brackets): FP32 with
+// a sphere 24^3 1 29.3, 2 29.1, 4 35.3, 6 41.5 [1]; 80 x 76 x 84 3 66, 4 53, 6 54,
+// 9 66 [4]; 128^3 4 123, 6 112, 8 109, 10 110, 12 115, 16 110 [10]; 256^3 8 668, 16
+// 610, 24 602, 32 602, 64 611 [32]; without one 64^3 2 37, 4 29, 8 31, 16 43 [4];
+// 80 x 76 x 84 4 58, 6 51, 9 47, 12 48, 24 59 [9]; FP64 32^3 1 133, 2 180, 6 377
+// [1]; 96^3 4 1092, 8 992, 12 994, 16 1197 [12]; 102 x 107 x 95 12 1609, 16 1827,
+// 19 1566, 24 1725 [19].
 int default_fused_planes(const DevParams& P, int halves)
 {
     const long long cols = (long long)((P.nx + 31) / 32) * ((P.ny + 7) / 8);
@@ -187,11 +188,12 @@ int default_fused_planes(const DevParams& P, int halves)
 
 // z chunk length of kz_scalars without lb_tune, by the same kind of model: 456
 // blocks at a time and five planes' time to start a block in FP32, the planes
-// of an SM's blocks in FP64.  Measured on GB300 (us, choice in brackets): FP32
-// 24^3 1 plane 13, 6 planes 21 [1]; 64^3 2 planes 14.7, 4 13.1, 16 17.1 [4];
-// 128^3 4 planes 56, 8 52, 12 50, 24 61 [8]; 256^3 8 planes 277, 24 250, 32 261,
-// 64 278 [32]; FP64 32^3 1 plane 63, 6 planes 140 [1]; 96^3 8 planes 428, 12
-// 406, 24 413 [12].
+// of an SM's blocks in FP64.  Measured on GB300 (us per launch, choice in
+// brackets): FP32 24^3 1 plane 13.0, 2 14.0, 6 18.8 [1]; 64^3 2 19.1, 4 16.7, 16
+// 26.4 [4]; 80 x 76 x 84 4 27, 6 24, 12 29 [6]; 128^3 4 56, 6 49, 8 51, 12 47, 24
+// 59 [8]; 256^3 8 270, 16 250, 24 247, 32 258, 64 268 [32]; FP64 32^3 1 65, 6 139
+// [1]; 96^3 8 468, 12 426, 16 544, 24 418 [12]; 102 x 107 x 95 6 687, 8 707, 12
+// 629, 16 790 [12].
 int default_scalar_planes(const DevParams& P, bool fp64)
 {
     const long long cols = (long long)((P.nx + 31) / 32) * ((P.ny + 7) / 8);
@@ -320,10 +322,13 @@ constexpr int kGraphSteps = 8, kGraphAfter = 128;
 // Whether graph launches beat plain ones.  Without particles they do (measured
 // on GB300: 170 instead of 174 us per step at 128^3).  With particles a step
 // has nine kernels on three streams; in a graph the edges between them cost
-// less, but the particle kernels lose some of their head start before the bulk
-// kernels.  Plain -> graph, us per step: FP32 24^3 70 -> 57, 40 x 38 x 44 71 ->
-// 61, 64^3 90 -> 84, 96^3 135 -> 118, 110 x 100 x 96 153 -> 156, 160 x 150 x 170
-// 283 -> 292; FP64 32^3 178 -> 172, 48^3 458 -> 482, 64^3 621 -> 617.
+// less, but the particle kernels may start later beside the bulk kernels.  Plain
+// -> graph, us per step with one sphere: FP32 24^3 52 -> 44, 48^3 68 -> 58, 64^3
+// 78 -> 74, 96^3 128 -> 117, 110 x 100 x 96 141 -> 139, 128^3 183 -> 180: the line
+// lies where two percent are left of the gain.  FP64 24^3 190 -> 184, 32^3 195 ->
+// 185, 33^3 320 -> 314, 40 x 38 x 44 339 -> 361, 44^3 464 -> 378, 48^3 490 -> 405,
+// 56^3 496 -> 488, 64^3 606 -> 613, 80^3 1154 -> 1138, 101^3 2167 -> 2157: up to
+// the line every measured box gains, above it most do and some lose.
 bool graph_pays(const DevParams& P, bool fp64) { return P.np == 0 || P.N <= (fp64 ? 1ll << 15 : 1ll << 20); }
 
 bool same_grid(const dim3& a, const dim3& b) { return a.x == b.x && a.y == b.y && a.z == b.z; }
